@@ -20,6 +20,7 @@
 // column and sweep the band with a register window (the interchanges stay inside it); the
 // reciprocal pivots are stored once, and the upper sweep runs at the bandwidth the
 // interchanges actually produced (15 when there were none).
+#include <algorithm>
 #include <cstdio>
 
 #include "spalu_internal.h"
@@ -918,6 +919,226 @@ __global__ void __launch_bounds__(SWPB * 32) leaf_solve_kernel(LeafDev d, T* X, 
   }
 }
 
+// ---- FP64 leaf sweeps over the band rows: few right-hand sides, or few leaves.
+//
+// A half-warp owns one leaf and its 16 lanes own the 16 rows of the sweep window (row j in lane
+// j mod 16), so a step is one shuffle and one multiply-add per right-hand side for all 15 rows
+// at once, instead of 15 multiply-adds in a thread that owns a whole column.  R right-hand sides
+// run side by side in a warp; the others are other warps (gridDim.y).
+// What bounds it: a FP64 warp instruction occupies an SM sub-partition for 64 cycles however few
+// of its lanes are active (measured: 64.1 cycles with 1 to 32 lanes, 67 from one to the next
+// that needs it).  Per two leaves and pair of steps (one of L, one of U) this form issues
+// 2 R + 1 of them for R right-hand sides, leaf_solve_kernel 31 for any number up to 16.
+// Forward + backward launch, before and after: 63^2, 1 right-hand side 294 + 314 -> 53 + 62 us;
+// 255^2, 5: 312 + 343 -> 62 + 72 us; 1023^2, 4: 894 + 1029 -> 340 + 386 us; with interchanges
+// (1023^2 Helmholtz, 8) 1959 + 2138 -> 1093 + 1235 us.
+// The U sweep scales the column by its reciprocal pivot (once per step, off the chain) instead of
+// the running value, and the solution rows once per 16 steps.
+// The right-hand sides (backward: A_Id x_d) are brought into shared memory first and the sweeps
+// run in place there; a lane reads and writes only rows j = lane mod 16, so the sweeps need no
+// barrier.  The records come straight from global memory, one block of 16 steps ahead (a
+// half-warp reads a record as one contiguous run).  Every address is valid whether or not its
+// value is used: shared loads under a condition may be issued ahead of it.
+constexpr int RWPB = 4;                                // warps per CTA
+constexpr int RNB = 15;                                // blocks of 16 rows (the last holds one)
+constexpr int RROW = 16 * (RNB + 1);                   // rows of a right-hand side and a block of zeros
+template <int R>
+__host__ __device__ constexpr int row_leaf_pitch() { return R * RROW + (R % 2 == 0 ? 16 : 0); }
+template <int R>
+__host__ __device__ constexpr size_t row_smem() { return (size_t)RWPB * 2 * row_leaf_pitch<R>() * sizeof(double); }
+
+// Records of block blk, lane l's slot of each: every address lies inside the leaf's records (the
+// last block repeats its one column, a block number past either end is clamped), so the loads
+// need no condition; the sweeps use only the columns that exist.
+__device__ __forceinline__ void rows_load_L(const double* lr, int blk, int l, double (&v)[16]) {
+  const int bk = min(max(blk, 0), RNB - 1);
+#pragma unroll
+  for (int u = 0; u < 16; ++u) v[u] = __ldg(lr + 16 * min(16 * bk + u, NI - 1) + ((l - u + 31) & 15));
+}
+__device__ __forceinline__ void rows_load_U(const double* ur, int blk, int l, double (&v)[16]) {
+  const int bk = min(max(blk, 0), RNB - 1);
+#pragma unroll
+  for (int u = 0; u < 16; ++u) v[u] = __ldg(ur + 16 * min(16 * bk + u, NI - 1) + ((u - l + 16) & 15));
+}
+
+// y = L^{-1} P y in place (y: R columns of RROW values, rows >= NI zero).  lv holds block 0.
+template <int R, bool PIV>
+__device__ __forceinline__ void rows_sweep_L(const double* lr, double* y, double (&lv)[16]) {
+  const int lane = threadIdx.x & 31, l = lane & 15, hb = lane & 16;
+  double W[R];
+#pragma unroll
+  for (int c = 0; c < R; ++c) W[c] = y[c * RROW + l];
+#pragma unroll 1
+  for (int blk = 0; blk < RNB; ++blk) {
+    double ln[16], nx[R], fin[R];
+    rows_load_L(lr, blk + 1, l, ln);
+#pragma unroll
+    for (int c = 0; c < R; ++c) {
+      nx[c] = y[c * RROW + 16 * (blk + 1) + l];        // past the last block: the zeros
+      fin[c] = 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+      if (16 * blk + u < NI) {
+        int dsw = 0;
+        if constexpr (PIV) dsw = (int)__shfl_sync(0xffffffffu, lv[u], hb | u);   // pivot offset 0..15
+        const double m = l == u ? 0.0 : lv[u];
+#pragma unroll
+        for (int c = 0; c < R; ++c) {
+          double b;
+          if constexpr (PIV) {
+            const int s = (u + dsw) & 15;
+            const double a = __shfl_sync(0xffffffffu, W[c], hb | u);
+            b = __shfl_sync(0xffffffffu, W[c], hb | s);
+            if (l == s) W[c] = a;                      // the interchanged row; lane u retires below
+          } else {
+            b = __shfl_sync(0xffffffffu, W[c], hb | u);
+          }
+          W[c] -= m * b;
+          if (l == u) { fin[c] = b; W[c] = nx[c]; }
+        }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < R; ++c) y[c * RROW + 16 * blk + l] = fin[c];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) lv[u] = ln[u];
+  }
+}
+
+// y = U^{-1} y in place; WIDE: upper bandwidth up to 30 (a second window of 16 rows).
+template <int R, bool WIDE>
+__device__ __forceinline__ void rows_sweep_U(const double* ur, const double* ux, double* y) {
+  const int lane = threadIdx.x & 31, l = lane & 15, hb = lane & 16;
+  constexpr int AHEAD = WIDE ? 2 : 1;
+  double uv[16], xv[16], V[R], V1[R];
+  rows_load_U(ur, RNB - 1, l, uv);
+  if constexpr (WIDE) rows_load_U(ux, RNB - 1, l, xv);
+  // the last block holds row NI - 1 (lane 0); the other lanes start one block down
+  const int top = l == 0 ? RNB - 1 : RNB - 2;
+#pragma unroll
+  for (int c = 0; c < R; ++c) {
+    V[c] = y[c * RROW + 16 * top + l];
+    V1[c] = WIDE ? y[c * RROW + 16 * (top - 1) + l] : 0.0;
+  }
+#pragma unroll 1
+  for (int blk = RNB - 1; blk >= 0; --blk) {
+    double un[16], xn[16], nx[R], fin[R], dself = 0.0;
+    rows_load_U(ur, blk - 1, l, un);
+    if constexpr (WIDE) rows_load_U(ux, blk - 1, l, xn);
+    // rows above the first do not exist: the zero block stands for them
+    const int nb = blk >= AHEAD ? blk - AHEAD : RNB;
+#pragma unroll
+    for (int c = 0; c < R; ++c) {
+      nx[c] = y[c * RROW + 16 * nb + l];
+      fin[c] = 0.0;
+    }
+#pragma unroll
+    for (int u = 15; u >= 0; --u) {
+      if (16 * blk + u < NI) {
+        const double dinv = __shfl_sync(0xffffffffu, uv[u], hb | u);
+        if (l == u) dself = uv[u];
+        const double g = l == u ? 0.0 : uv[u] * dinv;
+        double g1 = 0.0;
+        if constexpr (WIDE) g1 = xv[u] * dinv;         // slot r - 16; lane u: r = 16
+#pragma unroll
+        for (int c = 0; c < R; ++c) {
+          const double v = __shfl_sync(0xffffffffu, V[c], hb | u);
+          V[c] -= g * v;
+          if constexpr (WIDE) V1[c] -= g1 * v;
+          if (l == u) {
+            fin[c] = v;
+            if constexpr (WIDE) { V[c] = V1[c]; V1[c] = nx[c]; }
+            else V[c] = nx[c];
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < R; ++c) y[c * RROW + 16 * blk + l] = fin[c] * dself;   // rows >= NI stay zero
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+      uv[u] = un[u];
+      if constexpr (WIDE) xv[u] = xn[u];
+    }
+  }
+}
+
+template <int R, bool WIDE, bool bwd>
+__global__ void __launch_bounds__(RWPB * 32) leaf_rows_kernel(LeafDev d, double* X, int nrhs, VecLayout lay) {
+  extern __shared__ float4 lsm4[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane >> 4, l = lane & 15;
+  const int nbox = d.g.nbox();
+  // a warp without a leaf and a half-warp without one repeat the last leaf and store nothing
+  const int bq = (blockIdx.x * RWPB + warp) * 2 + sub;
+  const bool live = bq < nbox;
+  const int b = live ? bq : nbox - 1;
+  const int c0 = blockIdx.y * R;
+  double* y = reinterpret_cast<double*>(lsm4) + (2 * warp + sub) * row_leaf_pitch<R>();
+  const double* lr = reinterpret_cast<const double*>(d.lrec) + (size_t)b * NI * 16;
+  const double* ur = reinterpret_cast<const double*>(d.urec) + (size_t)b * NI * 16;
+  const double* ux = reinterpret_cast<const double*>(d.uext) + (size_t)b * NI * 16;
+  const int nx = d.nx;
+  const int o = (b % d.g.bx) * (LEAF + 1) + nx * ((b / d.g.bx) * (LEAF + 1));
+  double lv[16];
+  rows_load_L(lr, 0, l, lv);                           // the factor's: overlaps the preceding kernel
+  pdl_enter();
+  // rows l, l + 16, ... of the right-hand sides (backward: of A_Id x_d, the terms of a row in the
+  // order of the CSR columns; a coefficient of 0 may stand for a side outside the grid, and then
+  // the row's own node, which exists, is read and not used)
+#pragma unroll 1
+  for (int blk = 0; blk < RNB + 1; ++blk) {
+    const int jr = 16 * blk + l, j = min(jr, NI - 1);
+    const int lx = j % LEAF, ly = j / LEAF, own = o + lx + nx * ly;
+    const bool in = jr < NI;
+    double v[R];
+    if constexpr (!bwd) {
+#pragma unroll
+      for (int c = 0; c < R; ++c) {
+        const int cc = min(c0 + c, nrhs - 1);
+        const double xv = X[lay.at(own, cc)];
+        v[c] = (in && c0 + c < nrhs) ? xv : 0.0;
+      }
+    } else {
+      const double* cp = reinterpret_cast<const double*>(d.cpl) + (size_t)b * NQ;
+#pragma unroll
+      for (int c = 0; c < R; ++c) v[c] = 0.0;
+      auto term = [&](bool on, int q, int nb) {
+        const double a = on ? __ldg(cp + q) : 0.0;
+        if (a != 0.0) {
+#pragma unroll
+          for (int c = 0; c < R; ++c) {
+            const double xv = X[lay.at(nb, min(c0 + c, nrhs - 1))];
+            v[c] += a * xv;
+          }
+        }
+      };
+      if (in) {
+        term(ly == 0, lx, o - nx + lx);
+        term(lx == 0, 2 * LEAF + ly, o - 1 + nx * ly);
+        term(lx == LEAF - 1, 3 * LEAF + ly, o + LEAF + nx * ly);
+        term(ly == LEAF - 1, LEAF + lx, o + LEAF * nx + lx);
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < R; ++c) y[c * RROW + jr] = v[c];
+  }
+  rows_sweep_L<R, WIDE>(lr, y, lv);
+  rows_sweep_U<R, WIDE>(ur, ux, y);
+  if (!live) return;
+#pragma unroll 1
+  for (int j = l; j < NI; j += 16) {
+    const int node = o + j % LEAF + nx * (j / LEAF);
+#pragma unroll
+    for (int c = 0; c < R; ++c)
+      if (c0 + c < nrhs) {
+        double* x = X + lay.at(node, c0 + c);
+        if constexpr (!bwd) *x = y[c * RROW + j];
+        else *x -= y[c * RROW + j];
+      }
+  }
+}
+
 // Backward leaf step of the mixed path on grids of few leaves: x_I -= G x_d with
 // G = A_II^{-1} A_Id (FP32, stored by the factorization) and x_d the 60 side unknowns of the
 // leaf.  One leaf per CTA: G is staged in shared memory by cp.async while x_d is gathered,
@@ -1133,6 +1354,38 @@ static void leaf_solve_go(const LeafDev& d, T* X, int nrhs, VecLayout lay, int b
   }
 }
 
+template <int R, bool WIDE>
+static void leaf_rows_go(const LeafDev& d, double* X, int nrhs, VecLayout lay, int bwd, cudaStream_t s) {
+  const dim3 grid((d.g.nbox() + 2 * RWPB - 1) / (2 * RWPB), (nrhs + R - 1) / R);
+  const int smem = (int)row_smem<R>();
+  note_launch();
+  if (!bwd) {
+    cudaFuncSetAttribute(leaf_rows_kernel<R, WIDE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    launch_pdl(leaf_rows_kernel<R, WIDE, false>, grid, dim3(RWPB * 32), smem, s, d, X, nrhs, lay);
+  } else {
+    cudaFuncSetAttribute(leaf_rows_kernel<R, WIDE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    launch_pdl(leaf_rows_kernel<R, WIDE, true>, grid, dim3(RWPB * 32), smem, s, d, X, nrhs, lay);
+  }
+}
+
+// Right-hand sides per warp of the FP64 sweeps over the band rows, or 0 for the sweeps over columns
+// (leaf_solve_kernel).  Times in units of one FP64 warp instruction per step pair (7.2 us per
+// launch at 2 GHz): a form costs the larger of its latency with one warp per SM sub-partition and
+// its instructions x warps per sub-partition x the measured overhead of issuing them.  Measured
+// for 1 .. 16 right-hand sides on 31^2 .. 1023^2: the column form wins at 1023^2 from 12 up
+// (893 against 908 us forward) and at 511^2 at 16 (328 against 338 us), never below 511^2.
+static int leaf_rows_width(int nbox, int nrhs, bool wide) {
+  const double sub = 4.0 * sm_count(), pairs = (nbox + 1) / 2;
+  auto cost = [&](double lat, double instr, double over, double warps) {
+    return std::max(lat, instr * over * warps / sub);
+  };
+  const double col = wide ? cost(64, 46, 1.75, pairs) : cost(42, 31, 1.18, pairs);
+  const double r1 = wide ? cost(12, 5, 1.4, pairs * nrhs) : cost(7.4, 3, 1.4, pairs * nrhs);
+  const double r2 = wide ? cost(16, 8, 1.4, pairs * ((nrhs + 1) / 2)) : cost(11, 5, 1.4, pairs * ((nrhs + 1) / 2));
+  if (col <= r1 && col <= r2) return 0;
+  return r1 <= r2 ? 1 : 2;
+}
+
 // The FP32 solve vector is always chunked (VecLayout{16, 1, 16 N}: a node's 16 right-hand
 // sides contiguous, every chunk 64-byte aligned); the FP32 forward sweep stages its rows as such.
 void launch_leaf_solve(const LeafDev& d, void* Xv, int nrhs, VecLayout lay, int bwd, int kumax, cudaStream_t s) {
@@ -1155,7 +1408,12 @@ void launch_leaf_solve(const LeafDev& d, void* Xv, int nrhs, VecLayout lay, int 
       else leaf_solve_go<float, 32>(d, Xc, nc, lay, bwd, s);
     } else {
       double* Xc = static_cast<double*>(Xv) + (size_t)(c0 / SLOT) * lay.chunk;
-      if (kumax <= 15) leaf_solve_go<double, 16>(d, Xc, nc, lay, bwd, s);
+      const int R = leaf_rows_width(d.g.nbox(), nc, kumax > 15);
+      if (R == 1 && kumax <= 15) leaf_rows_go<1, false>(d, Xc, nc, lay, bwd, s);
+      else if (R == 1) leaf_rows_go<1, true>(d, Xc, nc, lay, bwd, s);
+      else if (R == 2 && kumax <= 15) leaf_rows_go<2, false>(d, Xc, nc, lay, bwd, s);
+      else if (R == 2) leaf_rows_go<2, true>(d, Xc, nc, lay, bwd, s);
+      else if (kumax <= 15) leaf_solve_go<double, 16>(d, Xc, nc, lay, bwd, s);
       else leaf_solve_go<double, 32>(d, Xc, nc, lay, bwd, s);
     }
   }
