@@ -81,7 +81,7 @@ typedef struct {
                                  holds) run at once on an SM; a segment that does not fit
                                  keeps its sketch rows in global memory (results agree up to
                                  rounding).  A level with at most one segment per SM gets
-                                 160 KB (room for larger sketch chunks and the staged
+                                 200 KB (room for larger sketch chunks and the staged
                                  neighbour block).  0 = size for the largest segment the
                                  geometry allows.  Default 4. */
   int schur_tc;               /* mixed precision only: 1 (default) = the separators' Schur

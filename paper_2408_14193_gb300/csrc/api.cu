@@ -726,10 +726,10 @@ spalu_status spalu_factor_create(spalu_nd_t nd, const spalu_opts* o, spalu_facto
     const int tb = o->precision == 1 ? 4 : 8;
     // need: the uncut working set with the smallest sketch chunk (below it the kernel keeps
     // its sketch rows in global scratch).  A level that runs one segment per SM (or the uncut
-    // candidate of the tuner) gets 160 KB: what a segment does not need for its working set
+    // candidate of the tuner) gets 200 KB: what a segment does not need for its working set
     // goes to larger sketch chunks and the staged B block
     size_t need = sparsify_smem_need(p.capS, o->symmetric, o->h0, o->p_oversample, tb, 16);
-    size_t lim = 160 * 1024;
+    size_t lim = 200 * 1024;
     size_t mn = sparsify_smem_min(p.capS, o->symmetric, o->h0, o->p_oversample, tb);
     const size_t roomy = std::max(lim, mn);
     const size_t full = std::min(need, roomy);
@@ -744,7 +744,14 @@ spalu_status spalu_factor_create(spalu_nd_t nd, const spalu_opts* o, spalu_facto
     p.spars_smem = full;
     if (o->spars_ctas > 0 && p.g.nseg() > 0) {
       const int nsm = sm_count();
-      p.spars_smem = budget((int)std::min<long long>(o->spars_ctas, ((long long)p.g.nseg() + nsm - 1) / nsm));
+      int ctas = (int)std::min<long long>(o->spars_ctas, ((long long)p.g.nseg() + nsm - 1) / nsm);
+      // ... but not so many that a usual segment (compressed sides reach about 40 unknowns) loses
+      // its working set to global scratch, which slows its QR threefold (FP64, 1023^2, level 9:
+      // 1.20 ms with four per SM, 0.8 with three)
+      const size_t usual = sparsify_smem_need(std::min(p.capS, 40), o->symmetric, o->h0, o->p_oversample, tb, 16) -
+                           sparsify_smem_stage(std::min(p.capS, 40), o->symmetric, tb);
+      while (ctas > 1 && budget(ctas) < std::min(full, usual)) --ctas;
+      p.spars_smem = budget(ctas);
     }
     size_t least = p.spars_smem;
     for (int c = 0; c < SPARS_NCAND; ++c) {
@@ -815,7 +822,10 @@ spalu_status spalu_factor_create(spalu_nd_t nd, const spalu_opts* o, spalu_facto
       d.T = real((size_t)nseg * p.capS * p.capS);
       d.Dm = real((size_t)nseg * p.capS * p.capS);
       d.Dinv = real((size_t)nseg * p.capS);
-      d.Yg = p.spars_global ? real((size_t)nseg * p.Ycap * p.capS) : nullptr;
+      // global sketch rows: for segments that outgrow the shared-memory budget, and to keep a sketch
+      // that a larger one continues (no segment within the rank bound is sketched twice)
+      const bool again = p.capS + o->p_oversample > 2 * o->h0;
+      d.Yg = p.spars_global || again ? real((size_t)nseg * p.Ycap * p.capS) : nullptr;
       Fst[l - 1] = real((size_t)p.gp.nbox() * p.ldFp * p.ldFp);
       d.Pinv = real((size_t)p.gp.nbox() * p.sepcap);
       d.F = Fst[l];

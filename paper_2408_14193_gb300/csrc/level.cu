@@ -21,6 +21,7 @@
 // GB300 runs FP64 at 2 FMA per clock per SM, so per-column scalars (Householder coefficients,
 // norm downdates) are computed once for 32 columns at a time (one lane per column) and
 // divisions are replaced by stored reciprocals.
+#include <algorithm>
 #include <cfloat>
 #include <cmath>
 
@@ -809,162 +810,495 @@ __device__ bool id_error_ok(const SegCtx& S, BGet bget, int halves, int e, int k
 }
 
 // ------------------------------------------------------------ sparsify: one CTA per segment
-// The same column-pivoted Householder QR for CTAs of NWT warps when e <= 64, with the row work
-// spread over the warps and the scalar work on warp 0; three barriers per step.  Lanes own
-// columns (lane l: columns l and l + 32), warps own rows (warp w: rows r = w mod NWT).  Per
-// step i: warp 0 downdates the FP64 squared norms by the row of step i - 1 (recomputing below
-// the guard), chooses the pivot and forms the Householder scalars from the pivot column
-// (before it moves), and publishes them; then every warp swaps columns i and p on its rows and
-// forms its partial dots v^T y_j over its rows; then every warp sums the partial dots in warp
-// order and updates its rows.  Same arithmetic as block_cpqr up to the order of the sums.
-// part: >= NWT * 64 values of T; pub: >= 4 values of T.  All threads call it.
-template <typename T, int NWT>
-__device__ int rows_cpqr(T* Y, int ldy, int m, int e, double eps, int* perm, T* part, T* pub, int* shi,
+// Barrier of the first QW warps of a CTA of NWT (all of them: the CTA's barrier).
+template <int QW, int NWT>
+__device__ __forceinline__ void qr_bar() {
+  if constexpr (QW == NWT) __syncthreads();
+  else asm volatile("bar.sync 1, %0;" ::"n"(QW * 32) : "memory");
+}
+
+__device__ __forceinline__ unsigned bits_hi(double x) { return (unsigned)((unsigned long long)dbits(x) >> 32); }
+__device__ __forceinline__ unsigned bits_lo(double x) { return (unsigned)(unsigned long long)dbits(x); }
+
+// normx = sqrt(s) of a positive s: in FP64 from the reciprocal square root (a division or square
+// root costs 6 to 10 dependent FP64 instructions of 67 cycles each)
+__device__ __forceinline__ float qr_norm(float s) { return sqrtf(s); }
+__device__ __forceinline__ double qr_norm(double s) { return s > 0.0 ? s * rsqrt(s) : 0.0; }
+
+// The pivot of a step, chosen by one warp: among its columns at positions >= i, the largest
+// squared norm, near-ties (TIE_RTOL) to the lowest position.  Norms are compared as bit patterns
+// (an FP64 comparison is an instruction of the FP64 pipe).  Returns the position; *col the column.
+template <int CS>
+__device__ __forceinline__ int qr_pivot(const double (&n1)[CS], const int (&pos)[CS], int i, int e, int* col) {
+  const int lane = threadIdx.x & 31;
+  const double tie = (1.0 - TIE_RTOL) * (1.0 - TIE_RTOL);   // on squared norms
+  unsigned hi = 0, lo = 0, best = 0xffffffffu;
+#pragma unroll
+  for (int t = 0; t < CS; ++t)
+    if (pos[t] >= i && pos[t] < e) hi = max(hi, bits_hi(n1[t]));
+  hi = __reduce_max_sync(0xffffffffu, hi);
+#pragma unroll
+  for (int t = 0; t < CS; ++t)
+    if (pos[t] >= i && pos[t] < e && bits_hi(n1[t]) == hi) lo = max(lo, bits_lo(n1[t]));
+  lo = __reduce_max_sync(0xffffffffu, lo);
+  const long long thr = dbits(__longlong_as_double(((long long)hi << 32) | lo) * tie);
+#pragma unroll
+  for (int t = 0; t < CS; ++t)
+    if (pos[t] >= i && pos[t] < e && dbits(n1[t]) >= thr) best = min(best, (unsigned)pos[t]);
+  best = __reduce_min_sync(0xffffffffu, best);
+  if (best >= (unsigned)e) best = (unsigned)i;   // only where a norm is not a number
+  *col = 0;
+#pragma unroll
+  for (int t = 0; t < CS; ++t) {
+    const unsigned b = __ballot_sync(0xffffffffu, pos[t] == (int)best);
+    if (b) *col = 32 * t + __ffs(b) - 1;
+  }
+  (void)lane;
+  return (int)best;
+}
+
+// Column-pivoted Householder QR for e <= 32 CS, on Y in place by the first QW warps (all threads
+// call it): pivot rule, truncation and kstop as in block_cpqr; norm downdates in FP64 with the
+// same guard, but where one column falls below it all norms are recomputed (they decay together, so
+// this happens two or three times per factorization instead of once or more per column).  Lanes
+// own columns (lane l: slots l, l + 32), warps own rows (r mod QW).  Columns are not interchanged:
+// a column's position in the pivot order is a register.  perm receives the columns by position,
+// slot their places: R(a, b) is Y[a + ldy slot[b]] on return (rows < k).  Once at most 32 columns
+// are left, those in slots 32 .. move to slots whose columns are done, and one set of lanes goes on.
+// What bounds it: the latency of a step, k steps in a row, and in FP64 the instructions of the
+// FP64 pipe (64 cycles each).  So a step has two barriers and one reduction: every warp applies the
+// previous reflection to its rows and, in the same pass, forms its partial products of the next
+// pivot column x with all columns (x itself among them); one warp sums them, d_j = x^T y_j, and
+// has the whole step from them: ||x||^2 = d_x, v^T y_j = d_j - alpha y_ij with v = x - alpha e_i, the
+// new row i of R, the norm downdates and the next pivot.  That warp differs between the CTAs of an
+// SM (rw), so that their FP64 chains do not meet on one sub-partition.
+// Measured per segment (1023^2, clock64, all passes) against the form with three phases, three
+// barriers and a norm recomputed per column: mixed 63 -> 30 us at level 11 (e ~ 21, four CTAs per
+// SM), 72 -> 36 us at level 7; FP64 (also with its working set in shared memory now)
+// 514 -> 101 us at level 11, 255 -> 162 us at level 6 (e ~ 37, one CTA per SM).
+// shr: 64 doubles (coef), then QW * 32 CS doubles (part); shi: >= 6.
+template <typename T, int NWT, int QW, int CS>
+__device__ int fast_cpqr(T* Y, int ldy, int m, int e, double eps, int* perm, int* slot, double* shr, int* shi,
                          int kstop) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int j = threadIdx.x; j < e; j += blockDim.x) perm[j] = j;
-  if (m == 0 || e == 0) { __syncthreads(); return 0; }
-  // initial squared norms: partial sums over each warp's rows, added in warp order by warp 0
-#pragma unroll
-  for (int t = 0; t < 2; ++t) {
-    const int j = lane + 32 * t;
-    T s = T(0);
-    if (j < e)
-      for (int r = warp; r < m; r += NWT) { const T v = Y[r + (size_t)ldy * j]; s += v * v; }
-    part[warp * 64 + j] = s;
+  constexpr int EC = 32 * CS;
+  if (m == 0 || e == 0) {
+    for (int j = threadIdx.x; j < e; j += blockDim.x) { perm[j] = j; slot[j] = j; }
+    __syncthreads();
+    return 0;
   }
-  __syncthreads();
-  const double tol3z = sqrt(DBL_EPSILON);
-  const double tie = (1.0 - TIE_RTOL) * (1.0 - TIE_RTOL);
+  T* coef = reinterpret_cast<T*>(shr);
+  T* part = reinterpret_cast<T*>(shr + 64);
+  double* part2 = shr + 64;                // the same place: norms, when they are recomputed
   const int kmax = min(min(m, e), kstop);
-  double n1[2] = {0.0, 0.0}, n2[2] = {0.0, 0.0};       // warp 0: squared norms of lane's columns
-  double ref = 0.0;
-  if (warp == 0) {
+  const int rw = (int)(blockIdx.x + blockIdx.x / 152u) & (QW - 1);
+  if (warp < QW) {
+    int pos[CS], id[CS];                   // position and original column of the lane's slots
+    T acc[CS];
+    T* yc[CS];                             // the slots (clamped: every address is valid)
+    double n1[CS], g2[CS];                 // warp rw: squared norm; sqrt(eps_64) times its reference
+    const double tol3z = sqrt(DBL_EPSILON);
+    int cs = CS;                           // sets of lanes with columns left
 #pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      T s = T(0);
-      for (int w = 0; w < NWT; ++w) s += part[w * 64 + lane + 32 * t];
-      n1[t] = n2[t] = lane + 32 * t < e ? (double)s : 0.0;
+    for (int t = 0; t < CS; ++t) {
+      const int j = lane + 32 * t;
+      pos[t] = id[t] = j;
+      acc[t] = T(0);
+      yc[t] = Y + ldy * min(j, e - 1);
+      n1[t] = g2[t] = 0.0;
+      if (j < e)
+        for (int r = warp; r < m; r += QW) { const T v = yc[t][r]; acc[t] += v * v; }
+      part[warp * EC + j] = acc[t];
     }
-  }
-  int k = kmax;
-  for (int i = 0; i < kmax; ++i) {
-    // ---- warp 0: downdates by row i - 1, pivot, Householder scalars of the pivot column
-    if (warp == 0) {
-      if (i > 0) {
-        unsigned fl = 0;
+    qr_bar<QW, NWT>();
+    if (warp == rw) {
 #pragma unroll
-        for (int t = 0; t < 2; ++t) {
+      for (int t = 0; t < CS; ++t) {
+        T s = T(0);
+        for (int w = 0; w < QW; ++w) s += part[w * EC + lane + 32 * t];
+        n1[t] = lane + 32 * t < e ? (double)s : 0.0;
+        g2[t] = tol3z * n1[t];
+      }
+      int pc;
+      const int pp = qr_pivot<CS>(n1, pos, 0, e, &pc);
+      if (lane == 0) { shi[0] = pc; shi[1] = pp; }
+    }
+    qr_bar<QW, NWT>();
+    int p = shi[0], pp = shi[1];           // pivot slot of the step and its position so far
+    T ref_eps = T(0);                      // warp rw: the truncation threshold eps |R_00|
+    bool dots = true;                      // the products of step i with column p are still to form
+    for (int i = 0;; ++i) {
+#pragma unroll
+      for (int t = 0; t < CS; ++t) {
+        const int j = lane + 32 * t;
+        if (j == p) pos[t] = i;
+        else if (pos[t] == i) pos[t] = pp;
+      }
+      if (dots) {
+        const T* yp = Y + ldy * p;
+#pragma unroll
+        for (int t = 0; t < CS; ++t) {
+          acc[t] = T(0);
+          if (t < cs && pos[t] >= i && pos[t] < e)
+#pragma unroll 2
+            for (int r = i + ((warp - i) & (QW - 1)); r < m; r += QW) acc[t] += yp[r] * yc[t][r];
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < CS; ++t) part[warp * EC + lane + 32 * t] = acc[t];
+      qr_bar<QW, NWT>();
+      if (warp == rw) {
+        T d[CS], yi[CS];
+#pragma unroll
+        for (int t = 0; t < CS; ++t) {
           const int j = lane + 32 * t;
-          if (j > i - 1 && j < e && n1[t] != 0.0) {
-            const double rij = (double)Y[(i - 1) + (size_t)ldy * j];
-            const double sn = fmax(n1[t] - rij * rij, 0.0);
-            if (sn <= tol3z * n2[t]) fl |= 1u << t;
-            else n1[t] = sn;
+          d[t] = yi[t] = T(0);
+          if (t < cs) {
+            T q[QW];
+#pragma unroll
+            for (int w = 0; w < QW; ++w) q[w] = part[w * EC + j];
+#pragma unroll
+            for (int o = QW / 2; o > 0; o >>= 1)
+#pragma unroll
+              for (int w = 0; w < o; ++w) q[w] += q[w + o];
+            d[t] = q[0];
+            yi[t] = yc[t][i];
           }
         }
-        unsigned f0 = __ballot_sync(0xffffffffu, fl & 1u), f1 = __ballot_sync(0xffffffffu, (fl >> 1) & 1u);
-        while (f0 | f1) {          // recompute from rows i.. (rare)
-          int j;
-          if (f0) { j = __ffs(f0) - 1; f0 &= f0 - 1; } else { j = 32 + __ffs(f1) - 1; f1 &= f1 - 1; }
-          double s2 = 0.0;
-          for (int r = i + lane; r < m; r += 32) { const double v = (double)Y[r + (size_t)ldy * j]; s2 += v * v; }
-          for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-          if (lane == (j & 31)) { if (j >> 5) { n1[1] = s2; n2[1] = s2; } else { n1[0] = s2; n2[0] = s2; } }
+        T dp = d[0], yp = yi[0];
+        if constexpr (CS == 2) { if (p >> 5) { dp = d[1]; yp = yi[1]; } }
+        const T s = __shfl_sync(0xffffffffu, dp, p & 31), x0 = __shfl_sync(0xffffffffu, yp, p & 31);
+        const T normx = qr_norm(s);
+        int stop = 0;
+        if (i == 0) {
+          if constexpr (sizeof(T) == 4) ref_eps = __double2float_rd(eps * (double)normx);   // exact test in T
+          else ref_eps = eps * normx;
+          if (normx == T(0)) stop = 2;
+        }
+        if (!stop && (normx <= ref_eps || normx == T(0))) stop = 1;
+        bool low = false;                  // some norm fell below the guard
+        int pn = 0, ppn = 0;
+        if (!stop) {
+          const T alpha = x0 >= T(0) ? -normx : normx;
+          const T v0 = x0 - alpha;
+          const T den = s + (x0 >= T(0) ? x0 : -x0) * normx;      // v^T v / 2
+          const T c2 = den > T(0) ? T(1) / den : T(0);
+#pragma unroll
+          for (int t = 0; t < CS; ++t) {
+            if (t < cs) {
+              const int j = lane + 32 * t;
+              const bool act = pos[t] > i && pos[t] < e;
+              const T cj = act ? c2 * (d[t] - alpha * yi[t]) : T(0);
+              const T rij = yi[t] - cj * v0;
+              coef[j] = cj;
+              if (act) {
+                yc[t][i] = rij;
+                if (dbits(n1[t]) != 0) {
+                  const double rd = (double)rij, sn = n1[t] - rd * rd;
+                  const long long sb = dbits(sn) < 0 ? 0 : dbits(sn);
+                  if (sb <= dbits(g2[t])) low = true;
+                  else n1[t] = __longlong_as_double(sb);
+                }
+              } else if (j == p) {
+                yc[t][i] = alpha;                                 // R_ii
+              }
+            }
+          }
+          low = __any_sync(0xffffffffu, low);
+          if (!low && i + 1 < kmax) ppn = qr_pivot<CS>(n1, pos, i + 1, e, &pn);
+        }
+        if (lane == 0) { shi[0] = pn; shi[1] = ppn; shi[2] = stop; shi[3] = low; }
+      }
+      qr_bar<QW, NWT>();
+      const int stop = shi[2], low = shi[3];
+      if (stop || i + 1 >= kmax) {
+        if (threadIdx.x == 0) shi[5] = stop == 2 ? 0 : stop == 1 ? i : kmax;
+        break;
+      }
+      const T* v = Y + ldy * p;            // the reflection's column (rows > i)
+      const int r0 = i + 1 + ((warp - i - 1) & (QW - 1));
+      T cj[CS];
+      bool act[CS];
+#pragma unroll
+      for (int t = 0; t < CS; ++t) {
+        act[t] = t < cs && pos[t] > i && pos[t] < e;
+        cj[t] = coef[lane + 32 * t];
+        acc[t] = T(0);
+      }
+      const bool shrink = CS == 2 && cs == 2 && e - i - 1 <= 32;
+      if (!low && !shrink) {
+        p = shi[0];
+        pp = shi[1];
+        const bool inset1 = p >= 32;
+#pragma unroll 4
+        for (int r = r0; r < m; r += QW) {
+          const T vr = v[r];
+          T y[CS];
+#pragma unroll
+          for (int t = 0; t < CS; ++t) {
+            y[t] = T(0);
+            if (act[t]) {
+              y[t] = yc[t][r] - cj[t] * vr;
+              yc[t][r] = y[t];
+            }
+          }
+          T yq = y[0];
+          if constexpr (CS == 2) { if (inset1) yq = y[1]; }
+          const T xr = __shfl_sync(0xffffffffu, yq, p & 31);
+#pragma unroll
+          for (int t = 0; t < CS; ++t)
+            if (act[t]) acc[t] += xr * y[t];
+        }
+        dots = false;
+        continue;
+      }
+      // the update alone (and the norms in FP64), then what precedes the next pivot's products
+      double a2[CS];
+#pragma unroll
+      for (int t = 0; t < CS; ++t) {
+        a2[t] = 0.0;
+        if (act[t])
+#pragma unroll 2
+          for (int r = r0; r < m; r += QW) {
+            const T y = yc[t][r] - cj[t] * v[r];
+            yc[t][r] = y;
+            if (low) a2[t] += (double)y * (double)y;
+          }
+      }
+      p = shi[0];
+      pp = shi[1];
+      if (low) {
+#pragma unroll
+        for (int t = 0; t < CS; ++t) part2[warp * EC + lane + 32 * t] = a2[t];
+        qr_bar<QW, NWT>();
+        if (warp == rw) {
+#pragma unroll
+          for (int t = 0; t < CS; ++t) {
+            if (t < cs) {
+              double q = part2[lane + 32 * t];
+              for (int w = 1; w < QW; ++w) q += part2[w * EC + lane + 32 * t];
+              if (act[t]) { n1[t] = q; g2[t] = tol3z * q; }
+            }
+          }
+          int pn;
+          const int ppn = qr_pivot<CS>(n1, pos, i + 1, e, &pn);
+          if (lane == 0) { shi[0] = pn; shi[1] = ppn; }
+        }
+        qr_bar<QW, NWT>();
+        p = shi[0];
+        pp = shi[1];
+      }
+      if constexpr (CS == 2) {
+        if (shrink) {
+          // at most 32 columns left: the x-th of those in slots 32 .. changes places with the x-th
+          // done column of slots 0 .. 31 (there are at least as many)
+          const unsigned mv = __ballot_sync(0xffffffffu, act[1]);
+          const unsigned fr = __ballot_sync(0xffffffffu, !act[0]);   // done (every slot < 32 exists)
+          qr_bar<QW, NWT>();                                         // all rows updated
+          const int src = act[1] ? __popc(mv & ((1u << lane) - 1u)) : -1;
+          int to = -1, from = -1;                                    // set 1 lane -> slot, set 0 slot <- lane
+          unsigned f = fr, g = mv;
+          for (int x = 0; g; ++x) {
+            const int a = __ffs(f) - 1, b = __ffs(g) - 1;
+            f &= f - 1;
+            g &= g - 1;
+            if (x % QW == warp) {
+              T* ya = Y + ldy * a;
+              T* yb = Y + ldy * (b + 32);
+              for (int r = lane; r < m; r += 32) { const T q = ya[r]; ya[r] = yb[r]; yb[r] = q; }
+            }
+            if (src == x) to = a;
+            if (lane == a) from = b;
+            if (p == b + 32) p = a;
+          }
+          // exchange the registers of the two sets (a lane gives its set 1 to the lane `to` and
+          // takes that lane's set 0)
+          const int pf = __shfl_sync(0xffffffffu, pos[1], from < 0 ? lane : from);
+          const int jf = __shfl_sync(0xffffffffu, id[1], from < 0 ? lane : from);
+          const double nf = __shfl_sync(0xffffffffu, n1[1], from < 0 ? lane : from);
+          const double gf = __shfl_sync(0xffffffffu, g2[1], from < 0 ? lane : from);
+          const int pt = __shfl_sync(0xffffffffu, pos[0], to < 0 ? lane : to);
+          const int jt = __shfl_sync(0xffffffffu, id[0], to < 0 ? lane : to);
+          if (to >= 0) { pos[1] = pt; id[1] = jt; }
+          if (from >= 0) { pos[0] = pf; id[0] = jf; n1[0] = nf; g2[0] = gf; }
+          cs = 1;
+          qr_bar<QW, NWT>();
         }
       }
-      long long mx = -1;
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        const int j = lane + 32 * t;
-        if (j >= i && j < e) mx = max(mx, dbits(n1[t]));
-      }
-      for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      const long long thr = dbits(__longlong_as_double(mx) * tie);
-      int p = e;
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        const int j = lane + 32 * t;
-        if (j >= i && j < e && dbits(n1[t]) >= thr && j < p) p = j;
-      }
-      for (int o = 16; o > 0; o >>= 1) p = min(p, __shfl_xor_sync(0xffffffffu, p, o));
-      if (p != i) {
-        const int si = i >> 5, sp = p >> 5;
-        const double i1 = __shfl_sync(0xffffffffu, si ? n1[1] : n1[0], i & 31);
-        const double i2 = __shfl_sync(0xffffffffu, si ? n2[1] : n2[0], i & 31);
-        const double p1 = __shfl_sync(0xffffffffu, sp ? n1[1] : n1[0], p & 31);
-        const double p2 = __shfl_sync(0xffffffffu, sp ? n2[1] : n2[0], p & 31);
-        if (lane == (i & 31)) { if (si) { n1[1] = p1; n2[1] = p2; } else { n1[0] = p1; n2[0] = p2; } }
-        if (lane == (p & 31)) { if (sp) { n1[1] = i1; n2[1] = i2; } else { n1[0] = i1; n2[0] = i2; } }
-        if (lane == 0) { const int t = perm[i]; perm[i] = perm[p]; perm[p] = t; }
-      }
-      const T* yp = Y + (size_t)ldy * p;
-      T s = T(0);
-      for (int r = i + lane; r < m; r += 32) { const T v = yp[r]; s += v * v; }
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) {
-        const T normx = sqrt(s);
-        const T x0 = yp[i];
-        const T alpha = x0 >= T(0) ? -normx : normx;
-        const T v0 = x0 - alpha;
-        const T vv = v0 * v0 + (s - x0 * x0);
-        if (i == 0) ref = (double)normx;
-        int stop = 0;
-        if (ref == 0.0) stop = 2;
-        else if ((double)normx <= eps * ref || normx == T(0)) stop = 1;
-        pub[0] = alpha;
-        pub[1] = v0;
-        pub[2] = vv > T(0) ? T(2) / vv : T(0);
-        shi[0] = p;
-        shi[1] = stop;
-      }
+      dots = true;
     }
-    __syncthreads();
-    const int p = shi[0], stop = shi[1];
-    // ---- every warp, its rows (one per lane): swap columns i and p (also on the stopping step,
-    //      as perm already has)
-    if (p != i)
-      for (int r = warp + NWT * lane; r < m; r += NWT * 32) {
-        T* a = Y + r + (size_t)ldy * i;
-        T* b = Y + r + (size_t)ldy * p;
-        const T tmp = *a; *a = *b; *b = tmp;
-      }
-    if (stop) { __syncthreads(); k = stop == 2 ? 0 : i; break; }
-    __syncwarp();
-    const T v0 = pub[1], c2 = pub[2];
-    // ---- every warp, its rows: partial dots with v (v_i = v0)
-    const int r0 = i + ((warp - i % NWT) + NWT) % NWT;   // this warp's first row >= i
-    T acc[2];
+    if (warp == rw) {
 #pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      const int j = lane + 32 * t;
-      acc[t] = T(0);
-      if (j > i && j < e) {
-        const T* yj = Y + (size_t)ldy * j;
-        const T* yi = Y + (size_t)ldy * i;
-        for (int r = r0; r < m; r += NWT) acc[t] += (r == i ? v0 : yi[r]) * yj[r];
-      }
-      part[warp * 64 + j] = acc[t];
+      for (int t = 0; t < CS; ++t)
+        if (lane + 32 * t < e) {
+          perm[pos[t]] = id[t];
+          slot[pos[t]] = lane + 32 * t;
+        }
     }
-    __syncthreads();
-    // ---- every warp, its rows: y_j -= c2 (v^T y_j) v
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      const int j = lane + 32 * t;
-      if (j > i && j < e) {
-        T d = T(0);
-        for (int w = 0; w < NWT; ++w) d += part[w * 64 + j];
-        const T cj = d * c2;
-        T* yj = Y + (size_t)ldy * j;
-        const T* yi = Y + (size_t)ldy * i;
-        for (int r = r0; r < m; r += NWT) yj[r] -= cj * (r == i ? v0 : yi[r]);
-      }
-    }
-    if (r0 == i && lane == 0) Y[i + (size_t)ldy * i] = pub[0];   // R_ii, by the warp owning row i
-    __syncthreads();
   }
   __syncthreads();
-  return k;
+  return shi[5];
+}
+
+// T (k x (e-k), ld ldt) = R_1^{-1} R_2 with R(a, b) = Y[a + ldy slot[b]] (k <= 64): four columns per
+// warp, lanes over the rows; the column of R_1 is scaled by its reciprocal pivot once for the four.
+// rinv: >= k scratch.
+template <typename T, int NWT>
+__device__ void fast_interp(const T* Y, int ldy, int k, int e, const int* slot, T* Tm, int ldt, T* rinv) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int CJ = 4;
+  for (int a = threadIdx.x; a < k; a += blockDim.x) rinv[a] = T(1) / Y[a + ldy * slot[a]];
+  __syncthreads();
+  for (int j0 = CJ * warp; j0 < e - k; j0 += CJ * NWT) {
+    T s[2][CJ];
+#pragma unroll
+    for (int q = 0; q < CJ; ++q) {
+      const int col = slot[min(k + j0 + q, e - 1)];
+#pragma unroll
+      for (int t = 0; t < 2; ++t) s[t][q] = lane + 32 * t < k ? Y[min(lane + 32 * t, k - 1) + ldy * col] : T(0);
+    }
+    for (int a = k - 1; a >= 0; --a) {
+      const T* ra = Y + ldy * slot[a];
+      const T iv = rinv[a];
+      T x[CJ];
+#pragma unroll
+      for (int q = 0; q < CJ; ++q) x[q] = __shfl_sync(0xffffffffu, a < 32 ? s[0][q] : s[1][q], a & 31);
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        if (lane + 32 * t < a) {
+          const T g = ra[lane + 32 * t] * iv;
+#pragma unroll
+          for (int q = 0; q < CJ; ++q) s[t][q] -= g * x[q];
+        }
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const int a = lane + 32 * t;
+      if (a < k) {
+#pragma unroll
+        for (int q = 0; q < CJ; ++q)
+          if (j0 + q < e - k) Tm[a + (size_t)ldt * (j0 + q)] = s[t][q] * rinv[a];
+      }
+    }
+  }
+  __syncthreads();
+}
+
+__device__ __forceinline__ unsigned abs_hi(double x) { return bits_hi(x) & 0x7fffffffu; }
+__device__ __forceinline__ unsigned abs_hi(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+__device__ __forceinline__ unsigned abs_lo(double x) { return bits_lo(x); }
+__device__ __forceinline__ unsigned abs_lo(float) { return 0u; }
+
+// Elimination of the last n = e - k rows and columns of the e x e block A (e <= 32 RS) with partial
+// pivoting among those rows: L, U and the multipliers in place (not interchanged afterwards),
+// W = L^{-1} P A_rk, Z = A_kr U^{-1} and A_kk - Z W, one pass per pivot: lanes own rows (lane l:
+// rows l, l + 32), warps own columns.  One barrier per pivot: the warp that holds the next pivot
+// column updates it first, finds its pivot, scales it (and the Z entries) and publishes both while
+// the others update the remaining columns.  piv, inv: n; shi: >= 4.  False on a zero pivot.
+// What bounds it: that chain (update, pivot search on bit patterns, one reciprocal, barrier); it
+// replaces five barriers per pivot and two serial sweeps for Z and the Schur update (1023^2, per
+// segment: FP64 33 -> 13 us at level 6, level 1 with e = 44 106 -> 41 us; mixed 18 -> 9, 54 -> 22 us).
+template <typename T, int NWT, int RS>
+__device__ bool fast_elim(T* A, int lda, int k, int e, int* piv, T* inv, int* shi, int* okf) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n = e - k;
+  // column cj = k + j of the block: pivot among rows >= cj, swap, scale rows below and rows < k
+  auto prepare = [&](int j) {
+    const int cj = k + j;
+    T* col = A + lda * cj;
+    T x[RS];
+    unsigned hi = 0, lo = 0, best = 0xffffffffu;
+#pragma unroll
+    for (int t = 0; t < RS; ++t) {
+      const int r = lane + 32 * t;
+      x[t] = r < e ? col[min(r, e - 1)] : T(0);
+      if (r >= cj && r < e) hi = max(hi, abs_hi(x[t]));
+    }
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if constexpr (sizeof(T) == 8) {
+#pragma unroll
+      for (int t = 0; t < RS; ++t) {
+        const int r = lane + 32 * t;
+        if (r >= cj && r < e && abs_hi(x[t]) == hi) lo = max(lo, abs_lo(x[t]));
+      }
+      lo = __reduce_max_sync(0xffffffffu, lo);
+    }
+#pragma unroll
+    for (int t = 0; t < RS; ++t) {
+      const int r = lane + 32 * t;
+      if (r >= cj && r < e && abs_hi(x[t]) == hi && abs_lo(x[t]) == lo) best = min(best, (unsigned)r);
+    }
+    best = __reduce_min_sync(0xffffffffu, best);
+    const int p = (int)min(best, (unsigned)(e - 1));
+    const bool zero = (hi | lo) == 0u;
+    const T pv = __shfl_sync(0xffffffffu, p < 32 ? x[0] : x[RS - 1], p & 31);
+    const T old = __shfl_sync(0xffffffffu, cj < 32 ? x[0] : x[RS - 1], cj & 31);
+    const T iv = zero ? T(0) : T(1) / pv;
+#pragma unroll
+    for (int t = 0; t < RS; ++t) {
+      const int r = lane + 32 * t;
+      if (r < e) {
+        if (r == cj) col[r] = pv;
+        else if (r > cj) col[r] = (r == p ? old : x[t]) * iv;
+        else if (r < k) col[r] = x[t] * iv;
+      }
+    }
+    if (lane == 0) {
+      shi[j & 1] = p;
+      piv[j] = p - k;
+      inv[j] = iv;
+      if (zero) *okf = 0;
+    }
+  };
+  if (threadIdx.x == 0) *okf = 1;
+  __syncthreads();
+  if (warp == 0) prepare(0);
+  __syncthreads();
+  for (int j = 0; j < n; ++j) {
+    const int cj = k + j, p = shi[j & 1];
+    T l[RS];
+    bool act[RS];
+#pragma unroll
+    for (int t = 0; t < RS; ++t) {
+      const int r = lane + 32 * t;
+      act[t] = r < e && (r < k || r > cj);
+      l[t] = act[t] ? A[min(r, e - 1) + lda * cj] : T(0);
+    }
+    // one column of the update: row cj takes row p's entry, row p the old row cj's
+    auto column = [&](int c) {
+      T* col = A + lda * c;
+      const T u = col[p], oc = col[cj];
+      T x[RS];
+#pragma unroll
+      for (int t = 0; t < RS; ++t) {
+        const int r = lane + 32 * t;
+        x[t] = act[t] ? (r == p ? oc : col[min(r, e - 1)]) - l[t] * u : u;
+      }
+      __syncwarp();
+#pragma unroll
+      for (int t = 0; t < RS; ++t) {
+        const int r = lane + 32 * t;
+        if (act[t] || r == cj) col[min(r, e - 1)] = x[t];
+      }
+      __syncwarp();
+    };
+    // columns 0 .. k-1 and cj+1 .. e-1; the next pivot column by warp (j + 1) mod NWT alone, the
+    // others by the other warps in turn
+    const int wn = (j + 1) % NWT;
+    const int nc = k + (n - j - 2 > 0 ? n - j - 2 : 0);
+    if (warp == wn && j + 1 < n) {
+      column(cj + 1);
+      prepare(j + 1);
+    } else {
+      const int nw = j + 1 < n ? NWT - 1 : NWT;
+      int w = warp;
+      if (j + 1 < n) w = (warp - wn - 1 + NWT) % NWT;      // 0 .. NWT-2
+      for (int x = w; x < nc; x += nw) column(x < k ? x : cj + 2 + (x - k));
+    }
+    __syncthreads();
+  }
+  return *okf != 0;
 }
 
 // Largest-first work list of a level (scheduling, not in the paper): a counting sort of the
@@ -998,6 +1332,13 @@ __global__ void __launch_bounds__(1024) seg_order_kernel(const int* cnt, int nse
   __syncthreads();
   for (int s = threadIdx.x; s < nseg; s += blockDim.x) order[atomicAdd(&start[key(cnt[s])], 1)] = s;
 }
+
+// Shared memory of a segment besides its blocks (norms, permutations, pivots, reciprocals), and the
+// values of its interpolation matrix (k (e - k) <= e^2 / 4, and room for the 8 probe rows)
+__host__ __device__ inline size_t sparsify_smem_small(int e, int tbytes) {
+  return 2 * (size_t)e * 8 + (3 * (size_t)e + 4) * 4 + (size_t)e * tbytes + 64;
+}
+__host__ __device__ inline int sparsify_t_values(int e) { return e * e / 4 > 8 * e ? e * e / 4 : 8 * e; }
 
 template <typename T, int NWT>
 __global__ void __launch_bounds__(NWT * 32, NWT == NW ? 4 : 16) sparsify_kernel(LevelDev d, int smem_bytes) {
@@ -1088,25 +1429,35 @@ __global__ void __launch_bounds__(NWT * 32, NWT == NW ? 4 : 16) sparsify_kernel(
   const int nF = halves * nfar_sh;
   const int hcap = max(d.h0, 2 * (e + d.p_over));
   const int hmax = min(nF, hcap);
-  const int mmax = nN + hmax;
+
+  // rank bound (k <= e): a segment with e + p <= 2 h0 is sketched once with
+  // h = min(2 h0, hmax) >= min(|F|, e + p), the size the adaptive schedule reaches at its
+  // second pass, and that pass always stands; the predictor serves the larger segments.
+  // Every h stays <= hbuf, the rows the sketch buffer was sized for.
+  const bool small = e + d.p_over <= 2 * d.h0;
+  const int hbuf = small ? min(hmax, 2 * d.h0) : hmax;
+  const int mmax = nN + hbuf;
 
   // working storage: vectors and sketch chunks in shared memory; Y, D, T too when they
-  // fit, else the global scratch of this segment
+  // fit, else the global scratch of this segment.  The sketch chunks and D share their place (D
+  // is formed when the last sketch is done), T holds k (e - k) values (or the 8 probe rows)
   const size_t TD = sizeof(T);
-  const size_t small_b = (2 * (size_t)e) * 8 + (3 * (size_t)e + 4) * 4 + (size_t)e * TD + 64;
-  const size_t per_ch_b = (size_t)halves * (e + hmax) * TD;
-  const size_t ydt_b = ((size_t)(mmax + 1) * e + 2 * (size_t)e * e) * TD;
+  const size_t small_b = sparsify_smem_small(e, (int)TD);
+  const size_t per_ch_b = (size_t)halves * (e + hbuf) * TD;
+  const size_t y_b = (size_t)(mmax + 1) * e * TD, t_b = (size_t)sparsify_t_values(e) * TD;
+  const size_t d_b = (size_t)e * e * TD;
+  auto fit_b = [&](int c) { return small_b + y_b + t_b + max(c * per_ch_b, d_b); };
   // chunk of the sketch product: the largest of 64, 32 and 16 far unknowns whose working set
   // fits the budget together with the staged B block (or without it, where B never fits):
   // fewer chunks, fewer barriers on the coarse levels' long far fields
   int ch = SK_CHUNK;
   {
     const size_t bsz = (size_t)halves * S.nb * e * TD + 48;
-    const bool keep_b = small_b + SK_CHUNK * per_ch_b + ydt_b + bsz <= (size_t)smem_bytes;
+    const bool keep_b = fit_b(SK_CHUNK) + bsz <= (size_t)smem_bytes;
     for (int c = SK_CHUNK_MAX; c > SK_CHUNK; c >>= 1)
-      if (small_b + c * per_ch_b + ydt_b + (keep_b ? bsz : 0) <= (size_t)smem_bytes) { ch = c; break; }
+      if (fit_b(c) + (keep_b ? bsz : 0) <= (size_t)smem_bytes) { ch = c; break; }
   }
-  bool in_smem = small_b + ch * per_ch_b + ydt_b <= (size_t)smem_bytes;
+  bool in_smem = fit_b(ch) <= (size_t)smem_bytes;
   if (!in_smem) {
     size_t room = (size_t)smem_bytes > small_b ? (size_t)smem_bytes - small_b : 0;
     ch = (int)min((size_t)SK_CHUNK, room / (per_ch_b > 0 ? per_ch_b : 1));
@@ -1116,7 +1467,7 @@ __global__ void __launch_bounds__(NWT * 32, NWT == NW ? 4 : 16) sparsify_kernel(
   bool bstage;
   double *vn1, *vn2;
   int *perm, *piv, *flags;
-  int ldy, ldd, ldt;
+  int ldy, ldd;
   {
     char* q = reinterpret_cast<char*>(sm);
     vn1 = reinterpret_cast<double*>(q); q += (size_t)e * 8;
@@ -1127,16 +1478,18 @@ __global__ void __launch_bounds__(NWT * 32, NWT == NW ? 4 : 16) sparsify_kernel(
     q = reinterpret_cast<char*>(((uintptr_t)q + 15) & ~(uintptr_t)15);
     rinv = reinterpret_cast<T*>(q); q += (size_t)e * TD;
     q = reinterpret_cast<char*>(((uintptr_t)q + 15) & ~(uintptr_t)15);
-    Bc = reinterpret_cast<T*>(q); q += (size_t)halves * ch * e * TD;
-    Gc = reinterpret_cast<T*>(q); q += (size_t)hmax * halves * ch * TD;
+    Bc = reinterpret_cast<T*>(q);
+    Gc = Bc + (size_t)halves * ch * e;
     if (in_smem) {
-      Y = reinterpret_cast<T*>(q); q += (size_t)(mmax + 1) * e * TD; ldy = mmax | 1;   // odd pitch
-      Dw = reinterpret_cast<T*>(q); q += (size_t)e * e * TD; ldd = e;
-      Tw = reinterpret_cast<T*>(q); q += (size_t)e * e * TD; ldt = e;
+      Dw = Bc; ldd = e;
+      q += max(ch * per_ch_b, d_b);
+      Y = reinterpret_cast<T*>(q); q += y_b; ldy = mmax | 1;   // odd pitch
+      Tw = reinterpret_cast<T*>(q); q += t_b;
     } else {
+      q += ch * per_ch_b;
       Y = static_cast<T*>(d.Yg) + (size_t)sid * d.Ycap * capS; ldy = d.Ycap;
       Dw = Dg; ldd = capS;
-      Tw = Tg; ldt = capS;
+      Tw = Tg;
     }
     // the segment's B block (every neighbour row, e columns) in what is left, when it fits
     q = reinterpret_cast<char*>(((uintptr_t)q + 15) & ~(uintptr_t)15);
@@ -1164,11 +1517,6 @@ __global__ void __launch_bounds__(NWT * 32, NWT == NW ? 4 : 16) sparsify_kernel(
   //      far rows, then the network's one-pass sketch size (PRED_PREDICT) or a training
   //      record of the features and the adaptive rank (PRED_RECORD)
   __shared__ float xf[PRED_NFEAT], zs[PRED_NFEAT], hid[PRED_NHID], pout[PRED_NOUT];
-  // rank bound (k <= e): a segment with e + p <= 2 h0 is sketched once with
-  // h = min(2 h0, hmax) >= min(|F|, e + p), the size the adaptive schedule reaches at its
-  // second pass, and that pass always stands; the predictor serves the larger segments.
-  // Every h stays <= hmax, the rows the sketch buffer was sized for.
-  const bool small = e + d.p_over <= 2 * d.h0;
   const bool use_pred = d.pred_mode != PRED_OFF && nF > max(d.h0, PRED_PROBE) && e <= PRED_EMAX && !small;
   int h = (nF <= d.h0) ? nF : small ? min(hmax, 2 * d.h0) : min(hmax, d.h0);
   bool predicted = false;
@@ -1193,11 +1541,18 @@ __global__ void __launch_bounds__(NWT * 32, NWT == NW ? 4 : 16) sparsify_kernel(
     }
   }
 
-  h = min(h, hmax);          // the sketch buffer holds nN + hmax rows
+  h = min(h, hbuf);          // the sketch buffer holds nN + hbuf rows
   // ---- adaptive sketch + ID (Sec. 4.2.3; h = k + p with k unknown: double h until k <= h - p)
   int k = 0;
   int passes = 0;
+  int ldt = capS;            // in shared memory: k
   bool fellback = false, have_t = false;
+  const bool fast = NWT != NW || e <= 64;   // the register-and-lane forms of the QR and what follows
+  // A pass that may have to be repeated with a larger h leaves its unscaled sketch rows in the
+  // segment's global scratch: the larger sketch has the same first rows (same counters, same
+  // sums), so only the new ones are formed
+  T* Ykeep = (in_smem && d.Yg) ? static_cast<T*>(d.Yg) + (size_t)sid * d.Ycap * capS : nullptr;
+  int have = 0;
   const bool was_predicted = predicted;
   unsigned long long work_done = 0;       // algorithmic FLOPs of this segment (thread 0)
   while (true) {
@@ -1230,31 +1585,40 @@ __global__ void __launch_bounds__(NWT * 32, NWT == NW ? 4 : 16) sparsify_kernel(
     } else {
       // Y_F = G B_F, chunks of neighbours (near ones get zero weight); the one-pass sketch of
       // a predicted segment takes its first PRED_PROBE rows from the probe
-      const int r0 = (predicted && e >= PRED_PROBE) ? min(PRED_PROBE, hh) : 0;
+      const bool probe = predicted && e >= PRED_PROBE;
+      const int r0 = probe ? min(PRED_PROBE, hh) : have;
       if (r0 < hh) sketch_far<T>(d, S, tb, bget, sid, halves, e, r0, hh, Y + nN, ldy, Bc, Gc, ch);
       const T sc = (T)(1.0 / sqrt((double)hh));
+      const bool keep = Ykeep && (predicted || e > hh - d.p_over);
       for (int x = threadIdx.x; x < hh * e; x += blockDim.x) {
         const int rr = x % hh, c = x / hh;
         T* yv = Y + (nN + rr) + (size_t)ldy * c;
-        *yv = (rr < r0 ? Tw[rr + PRED_PROBE * c] : *yv) * sc;
+        const T v = rr >= r0 ? *yv : probe ? Tw[rr + PRED_PROBE * c] : Ykeep[rr + (size_t)d.Ycap * c];
+        if (keep && rr >= have) Ykeep[rr + (size_t)d.Ycap * c] = v;
+        *yv = v * sc;
       }
+      if (keep) have = hh & ~3;              // whole counters of four rows
     }
     __syncthreads();
     // a pass that can still double h only needs to know whether k > h - p: its QR stops at
     // step h - p + 1 (the same decision, the remaining steps skipped)
     const int kstop = (!full && h < nF) ? max(1, hh - d.p_over + 1) : e;
-    k = (NWT == NW && e <= 64)
-            ? rows_cpqr<T, NWT>(Y, ldy, m, e, d.eps, perm, reinterpret_cast<T*>(shr),
-                                reinterpret_cast<T*>(shr) + NWT * 64, shi, kstop)
-            : block_cpqr<T, NWT>(Y, ldy, m, e, d.eps, perm, vn1, vn2, shr, flags, shi, kstop);
+    {
+      constexpr int QW = NWT != NW ? NWT : sizeof(T) == 8 ? 4 : 8;
+      if (!fast) k = block_cpqr<T, NWT>(Y, ldy, m, e, d.eps, perm, vn1, vn2, shr, flags, shi, kstop);
+      else if (NWT != NW || e <= 32) k = fast_cpqr<T, NWT, QW, 1>(Y, ldy, m, e, d.eps, perm, flags, shr, shi, kstop);
+      else if constexpr (NWT == NW) k = fast_cpqr<T, NWT, QW, 2>(Y, ldy, m, e, d.eps, perm, flags, shr, shi, kstop);
+    }
     ++passes;
     if (threadIdx.x == 0) work_done += work::qr(m, e, k);
+    if (in_smem) ldt = max(k, 1);
     if (predicted) {          // the one-pass ID stands if it passes the measured-error test
       predicted = false;
       if (full) break;
       bool ok = k <= h - d.p_over;
       if (ok) {
-        block_interp<T>(Y, ldy, k, e, Tw, ldt, rinv);
+        if (fast) fast_interp<T, NWT>(Y, ldy, k, e, flags, Tw, ldt, rinv);
+        else block_interp<T>(Y, ldy, k, e, Tw, ldt, rinv);
         have_t = true;
         ok = id_error_ok<T>(S, bget, halves, e, k, perm, Tw, ldt, d.eps, shr);
       }
@@ -1282,7 +1646,10 @@ __global__ void __launch_bounds__(NWT * 32, NWT == NW ? 4 : 16) sparsify_kernel(
     }
   }
   const int r = e - k;
-  if (!have_t) block_interp<T>(Y, ldy, k, e, Tw, ldt, rinv);
+  if (!have_t) {
+    if (fast) fast_interp<T, NWT>(Y, ldy, k, e, flags, Tw, ldt, rinv);
+    else block_interp<T>(Y, ldy, k, e, Tw, ldt, rinv);
+  }
 
   // ---- transformed diagonal block in [skeleton | remainder] order (Eq. (UtALt))
   for (int x = threadIdx.x; x < e * e; x += blockDim.x) {
@@ -1311,7 +1678,12 @@ __global__ void __launch_bounds__(NWT * 32, NWT == NW ? 4 : 16) sparsify_kernel(
   }
   // ---- eliminate the remainder: LU(A_rr) with W = L^{-1} P A_rk, Z = A_kr U^{-1},
   //      A_kk -= Z W  (Eq. (L^-1 * A * U^-1) for the segments of level l)
-  if (r > 0) {
+  if (r > 0 && fast) {
+    bool ok;
+    if (NWT != NW || e <= 32) ok = fast_elim<T, NWT, 1>(Dw, ldd, k, e, piv, rinv, shi, shi + 6);
+    else ok = fast_elim<T, NWT, 2>(Dw, ldd, k, e, piv, rinv, shi, shi + 6);
+    if (!ok && threadIdx.x == 0) atomicOr(d.err, ERR_SINGULAR);
+  } else if (r > 0) {
     bool ok = block_gepp<T>(Dw, ldd, k, r, e, piv, rinv, shi);
     if (!ok && threadIdx.x == 0) atomicOr(d.err, ERR_SINGULAR);
     if (k > 0) {
@@ -2281,20 +2653,26 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 16) sep_solve_kernel(Level
 
 }  // namespace
 
+// The sizes below follow the layout of sparsify_kernel.
 size_t sparsify_smem_need(int e, int symmetric, int h0, int p_over, int tbytes, int chunk) {
   const size_t halves = symmetric ? 1 : 2;
   const size_t hcap = (size_t)(h0 > 2 * (e + p_over) ? h0 : 2 * (e + p_over));
   const size_t mmax = halves * NEAR_MAX + hcap;
-  const size_t small_b = 2 * (size_t)e * 8 + (3 * (size_t)e + 4) * 4 + (size_t)e * tbytes + 64;
-  // segments of at most 32 unknowns also stage their B block (<= 6 sides of e + 8 corners)
-  const size_t bs = e <= 32 ? halves * (6 * (size_t)e + 8) * e + 4 : 0;
-  return small_b + ((size_t)chunk * halves * (e + hcap) + (mmax + 1) * e + 2 * (size_t)e * e + bs) * tbytes;
+  const size_t un = std::max((size_t)chunk * halves * (e + hcap), (size_t)e * e);
+  return sparsify_smem_small(e, tbytes) + (un + (mmax + 1) * e + sparsify_t_values(e)) * tbytes +
+         sparsify_smem_stage(e, symmetric, tbytes);
+}
+
+// segments of at most 32 unknowns also stage their B block (<= 6 sides of e + 8 corners)
+size_t sparsify_smem_stage(int e, int symmetric, int tbytes) {
+  const size_t halves = symmetric ? 1 : 2;
+  return e <= 32 ? (halves * (6 * (size_t)e + 8) * e + 4) * tbytes : 0;
 }
 
 size_t sparsify_smem_min(int e, int symmetric, int h0, int p_over, int tbytes) {
   const size_t halves = symmetric ? 1 : 2;
   const size_t hcap = (size_t)(h0 > 2 * (e + p_over) ? h0 : 2 * (e + p_over));
-  return 2 * (size_t)e * 8 + (3 * (size_t)e + 4) * 4 + (size_t)e * tbytes + 64 + halves * (e + hcap) * tbytes;
+  return sparsify_smem_small(e, tbytes) + halves * (e + hcap) * tbytes;
 }
 
 int sm_count() {
