@@ -39,6 +39,7 @@ constexpr int SK_CHUNK_MAX = 64;  // ... and at most, where the shared-memory bu
 constexpr int NW = 8;             // warps per CTA of the sparsify kernel (segments with e > 32)
 constexpr int NW_SMALL = 2;       // ... and for levels whose segments have at most 16 unknowns
 constexpr double TIE_RTOL = 1e-12;
+constexpr int INV_MAX = 64;       // triangular blocks up to this order are stored inverted (see below)
 constexpr int RSTAGE = 96;        // triangular blocks up to this order are staged in shared memory
 
 // ------------------------------------------------------------ Philox4x32-10 (SC'11)
@@ -400,11 +401,11 @@ __device__ void block_interp(const T* Y, int ldy, int k, int e, T* Tm, int ldt, 
 
 // LU with partial pivoting of the n x n block of A at (r0, r0) (ld lda), with the row
 // operations carried over columns [0, ncol) outside the factored block; multipliers are
-// stored below the diagonal and not interchanged afterwards (the solve interleaves
+// stored below the diagonal and (unless `all`) not interchanged afterwards (the solve interleaves
 // interchanges and eliminations).  inv receives the reciprocal pivots.  Returns false on an
 // exactly zero pivot.
 template <typename T>
-__device__ bool block_gepp(T* A, int lda, int r0, int n, int ncol, int* piv, T* inv, int* shi) {
+__device__ bool block_gepp(T* A, int lda, int r0, int n, int ncol, int* piv, T* inv, int* shi, bool all) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   bool ok = true;
   for (int j = 0; j < n; ++j) {
@@ -428,7 +429,7 @@ __device__ bool block_gepp(T* A, int lda, int r0, int n, int ncol, int* piv, T* 
     if (shi[1]) { ok = false; if (threadIdx.x == 0) inv[j] = T(0); __syncthreads(); continue; }
     if (p != j) {
       for (int c = threadIdx.x; c < ncol; c += blockDim.x) {
-        if (c >= r0 && c < cj) continue;
+        if (!all && c >= r0 && c < cj) continue;
         T a = A[(r0 + j) + (size_t)lda * c];
         A[(r0 + j) + (size_t)lda * c] = A[(r0 + p) + (size_t)lda * c];
         A[(r0 + p) + (size_t)lda * c] = a;
@@ -1191,16 +1192,17 @@ __device__ __forceinline__ unsigned abs_lo(double x) { return bits_lo(x); }
 __device__ __forceinline__ unsigned abs_lo(float) { return 0u; }
 
 // Elimination of the last n = e - k rows and columns of the e x e block A (e <= 32 RS) with partial
-// pivoting among those rows: L, U and the multipliers in place (not interchanged afterwards),
+// pivoting among those rows: L, U and the multipliers in place (interchanged with their rows),
 // W = L^{-1} P A_rk, Z = A_kr U^{-1} and A_kk - Z W, one pass per pivot: lanes own rows (lane l:
 // rows l, l + 32), warps own columns.  One barrier per pivot: the warp that holds the next pivot
 // column updates it first, finds its pivot, scales it (and the Z entries) and publishes both while
-// the others update the remaining columns.  piv, inv: n; shi: >= 4.  False on a zero pivot.
+// the others update the remaining columns.  q receives the permutation ((P b)_i = b_{q_i}), inv
+// the reciprocal pivots: n each; shi: >= 4.  False on a zero pivot.
 // What bounds it: that chain (update, pivot search on bit patterns, one reciprocal, barrier); it
 // replaces five barriers per pivot and two serial sweeps for Z and the Schur update (1023^2, per
 // segment: FP64 33 -> 13 us at level 6, level 1 with e = 44 106 -> 41 us; mixed 18 -> 9, 54 -> 22 us).
 template <typename T, int NWT, int RS>
-__device__ bool fast_elim(T* A, int lda, int k, int e, int* piv, T* inv, int* shi, int* okf) {
+__device__ bool fast_elim(T* A, int lda, int k, int e, int* q, T* inv, int* shi, int* okf) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n = e - k;
   // column cj = k + j of the block: pivot among rows >= cj, swap, scale rows below and rows < k
@@ -1246,12 +1248,15 @@ __device__ bool fast_elim(T* A, int lda, int k, int e, int* piv, T* inv, int* sh
     }
     if (lane == 0) {
       shi[j & 1] = p;
-      piv[j] = p - k;
+      const int a = q[j], b = q[p - k];
+      q[j] = b;
+      q[p - k] = a;
       inv[j] = iv;
       if (zero) *okf = 0;
     }
   };
   if (threadIdx.x == 0) *okf = 1;
+  for (int j = threadIdx.x; j < n; j += blockDim.x) q[j] = j;
   __syncthreads();
   if (warp == 0) prepare(0);
   __syncthreads();
@@ -1283,6 +1288,13 @@ __device__ bool fast_elim(T* A, int lda, int k, int e, int* piv, T* inv, int* sh
       }
       __syncwarp();
     };
+    // the multipliers of earlier steps follow their rows
+    if (p != cj)
+      for (int c = k + threadIdx.x; c < cj; c += blockDim.x) {
+        const T a = A[cj + lda * c];
+        A[cj + lda * c] = A[p + lda * c];
+        A[p + lda * c] = a;
+      }
     // columns 0 .. k-1 and cj+1 .. e-1; the next pivot column by warp (j + 1) mod NWT alone, the
     // others by the other warps in turn
     const int wn = (j + 1) % NWT;
@@ -1299,6 +1311,75 @@ __device__ bool fast_elim(T* A, int lda, int k, int e, int* piv, T* inv, int* sh
     __syncthreads();
   }
   return *okf != 0;
+}
+
+// X (n x n, ld n) = [L^{-1} \ U^{-1}] of the factored n x n block A (ld lda, n <= 32 RS; unit lower
+// L below the diagonal, reciprocal pivots rinv): the solve applies the two as products.  Four
+// columns per warp, lanes over the rows, one step per row of the block; U is scaled by the
+// reciprocal pivot of the step once for the four columns.
+template <typename T, int NWT, int RS>
+__device__ void fast_invert(const T* A, int lda, int n, const T* rinv, T* X) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int CJ = 4;
+  for (int j0 = CJ * warp; j0 < n; j0 += CJ * NWT) {
+    T s[RS][CJ];
+#pragma unroll
+    for (int t = 0; t < RS; ++t)
+#pragma unroll
+      for (int q = 0; q < CJ; ++q) {
+        const int i = lane + 32 * t, j = j0 + q;
+        const T v = A[min(i, n - 1) + lda * min(j, n - 1)];
+        s[t][q] = (i > j && i < n) ? v : T(0);
+      }
+    for (int m = j0 + 1; m < n; ++m) {             // L x = e_j: x_i = -(L_ij + sum_m L_im x_m)
+      T x[CJ];
+#pragma unroll
+      for (int q = 0; q < CJ; ++q) x[q] = __shfl_sync(0xffffffffu, m < 32 ? s[0][q] : s[RS - 1][q], m & 31);
+#pragma unroll
+      for (int t = 0; t < RS; ++t) {
+        const int i = lane + 32 * t;
+        if (i > m && i < n) {
+          const T l = A[i + lda * m];
+#pragma unroll
+          for (int q = 0; q < CJ; ++q) s[t][q] -= l * x[q];
+        }
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < RS; ++t)
+#pragma unroll
+      for (int q = 0; q < CJ; ++q) {
+        const int i = lane + 32 * t, j = j0 + q;
+        if (i > j && i < n) X[i + n * j] = -s[t][q];
+        s[t][q] = T(0);
+      }
+    for (int m = min(j0 + CJ, n) - 1; m >= 0; --m) {   // U x = e_j: x_i = -rinv_i sum_{m > i} U_im x_m
+      T x[CJ];
+#pragma unroll
+      for (int q = 0; q < CJ; ++q) {
+        x[q] = __shfl_sync(0xffffffffu, m < 32 ? s[0][q] : s[RS - 1][q], m & 31);
+        if (m == j0 + q) x[q] = T(-1);
+      }
+      const T iv = rinv[m];
+#pragma unroll
+      for (int t = 0; t < RS; ++t) {
+        const int i = lane + 32 * t;
+        if (i < m) {
+          const T g = A[i + lda * m] * iv;
+#pragma unroll
+          for (int q = 0; q < CJ; ++q) s[t][q] -= g * x[q];
+        }
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < RS; ++t)
+#pragma unroll
+      for (int q = 0; q < CJ; ++q) {
+        const int i = lane + 32 * t, j = j0 + q;
+        if (i <= j && j < n) X[i + n * j] = i == j ? rinv[i] : -s[t][q] * rinv[i];
+      }
+  }
+  __syncthreads();
 }
 
 // Largest-first work list of a level (scheduling, not in the paper): a counting sort of the
@@ -1444,7 +1525,7 @@ __global__ void __launch_bounds__(NWT * 32, NWT == NW ? 4 : 16) sparsify_kernel(
   const size_t TD = sizeof(T);
   const size_t small_b = sparsify_smem_small(e, (int)TD);
   const size_t per_ch_b = (size_t)halves * (e + hbuf) * TD;
-  const size_t y_b = (size_t)(mmax + 1) * e * TD, t_b = (size_t)sparsify_t_values(e) * TD;
+  const size_t y_b = (size_t)max(mmax + 1, e) * e * TD, t_b = (size_t)sparsify_t_values(e) * TD;
   const size_t d_b = (size_t)e * e * TD;
   auto fit_b = [&](int c) { return small_b + y_b + t_b + max(c * per_ch_b, d_b); };
   // chunk of the sketch product: the largest of 64, 32 and 16 far unknowns whose working set
@@ -1684,7 +1765,7 @@ __global__ void __launch_bounds__(NWT * 32, NWT == NW ? 4 : 16) sparsify_kernel(
     else ok = fast_elim<T, NWT, 2>(Dw, ldd, k, e, piv, rinv, shi, shi + 6);
     if (!ok && threadIdx.x == 0) atomicOr(d.err, ERR_SINGULAR);
   } else if (r > 0) {
-    bool ok = block_gepp<T>(Dw, ldd, k, r, e, piv, rinv, shi);
+    bool ok = block_gepp<T>(Dw, ldd, k, r, e, piv, rinv, shi, r <= INV_MAX);
     if (!ok && threadIdx.x == 0) atomicOr(d.err, ERR_SINGULAR);
     if (k > 0) {
       for (int a = threadIdx.x; a < k; a += blockDim.x) {     // Z = A_kr U^{-1}, row by row
@@ -1703,6 +1784,19 @@ __global__ void __launch_bounds__(NWT * 32, NWT == NW ? 4 : 16) sparsify_kernel(
       }
       __syncthreads();
     }
+  }
+  // ---- the remainder block inverted for the solve (the sketch's place is free), r <= INV_MAX
+  if (r > 0 && r <= INV_MAX) {
+    T* Db = Dw + k + (size_t)ldd * k;
+    if (NWT != NW || r <= 32) fast_invert<T, NWT, 1>(Db, ldd, r, rinv, Y);
+    else fast_invert<T, NWT, 2>(Db, ldd, r, rinv, Y);
+    for (int x = threadIdx.x; x < r * r; x += blockDim.x) Db[(x % r) + (size_t)ldd * (x / r)] = Y[x];
+    if (!fast && threadIdx.x == 0) {     // the pivot sequence as a permutation
+      for (int i = 0; i < r; ++i) flags[i] = i;
+      for (int j = 0; j < r; ++j) { const int p = piv[j], t = flags[j]; flags[j] = flags[p]; flags[p] = t; }
+      for (int i = 0; i < r; ++i) piv[i] = flags[i];
+    }
+    __syncthreads();
   }
   // ---- outputs
   if (in_smem) {
@@ -1922,117 +2016,13 @@ __global__ void merge_assemble_kernel(LevelDev d) {
   }
 }
 
-// LU of the separator block with the row operations over every column (W = L^{-1} P A_pd),
-// then Z = A_dp U^{-1}.  When the kp separator rows over all nM columns fit in the dynamic
-// shared memory (smem_bytes), they are staged there: the elimination then runs on shared
-// memory with the same operations in the same order, and the rows are written back once.
-template <typename T, bool ZREG>
-__global__ void __launch_bounds__(256) merge_panel_kernel(LevelDev d, int smem_bytes) {
-  extern __shared__ double pm_sm[];
-  __shared__ int shi[4];
-  const int P = blockIdx.x;
-  const int ndP = d.pcount[2 * P], kp = d.pcount[2 * P + 1];
-  if (kp == 0) return;
-  const int nM = ndP + kp;
-  const int* tab = d.ptab + (size_t)P * d.ldFp * TABW;
+// Separators of more than INV_MAX unknowns: LU of the separator block in global memory with the
+// row operations over every column (W = L^{-1} P A_pd), then Z = A_dp U^{-1}; one CTA.
+template <typename T>
+__device__ void panel_large(const LevelDev& d, T* M, const int* tab, int ndP, int kp, int* piv, T* inv, int* shi) {
+  const int nM = ndP + kp, Dp = d.gp.D();
   const size_t ldp = d.ldFp;
-  T* M = static_cast<T*>(d.Fp) + (size_t)P * ldp * ldp;
-  T* inv = static_cast<T*>(d.Pinv) + (size_t)P * d.sepcap;
-  const int Dp = d.gp.D();
-  int* piv = d.ppiv + (size_t)P * d.sepcap;
   bool ok = true;
-  if ((size_t)kp * nM * sizeof(T) + (size_t)nM * sizeof(int) <= (size_t)smem_bytes) {
-    // staged rows: Pn[r + kp c] = M[Dp + r, column of table entry c]; entries [ndP, nM) are
-    // the separator itself (positions Dp + j), [0, ndP) the parent boundary
-    T* Pn = reinterpret_cast<T*>(pm_sm);
-    int* colp = reinterpret_cast<int*>(Pn + (size_t)kp * nM);
-    for (int c = threadIdx.x; c < nM; c += blockDim.x) colp[c] = tab[(size_t)c * TABW];
-    __syncthreads();
-    for (int x = threadIdx.x; x < kp * nM; x += blockDim.x)
-      Pn[x] = M[(Dp + x % kp) + ldp * colp[x / kp]];
-    __syncthreads();
-    auto at = [&](int r, int c) -> T& { return Pn[r + (size_t)kp * c]; };
-    for (int j = 0; j < kp; ++j) {
-      const int cs = ndP + j;                   // staged column of separator unknown j
-      if (threadIdx.x < 32) {
-        int lane = threadIdx.x;
-        double best = -1.0;
-        int bi = kp;
-        for (int r = j + lane; r < kp; r += 32) {
-          double v = fabs((double)at(r, cs));
-          if (v > best || (v == best && r < bi)) { best = v; bi = r; }
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-          double ob = __shfl_xor_sync(0xffffffffu, best, o);
-          int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-          if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-        }
-        if (lane == 0) { shi[0] = bi; shi[1] = best == 0.0; piv[j] = bi; }
-      }
-      __syncthreads();
-      const int p = shi[0];
-      if (shi[1]) { ok = false; if (threadIdx.x == 0) inv[j] = T(0); __syncthreads(); continue; }
-      if (p != j) {
-        for (int c = threadIdx.x; c < nM; c += blockDim.x) {
-          if (c >= ndP && c < cs) continue;     // multipliers of earlier steps
-          T a = at(j, c);
-          at(j, c) = at(p, c);
-          at(p, c) = a;
-        }
-        __syncthreads();
-      }
-      const T ipv = T(1) / at(j, cs);
-      if (threadIdx.x == 0) inv[j] = ipv;
-      for (int r = j + 1 + threadIdx.x; r < kp; r += blockDim.x) at(r, cs) *= ipv;
-      __syncthreads();
-      const int nr = kp - j - 1;
-      const int ncols = (kp - j - 1) + ndP;
-      for (int x = threadIdx.x; x < nr * ncols; x += blockDim.x) {
-        int r = j + 1 + x % nr, cc = x / nr;
-        int c = cc < kp - j - 1 ? (cs + 1 + cc) : (cc - (kp - j - 1));
-        at(r, c) -= at(r, cs) * at(j, c);
-      }
-      __syncthreads();
-    }
-    if (!ok && threadIdx.x == 0) atomicOr(d.err, ERR_SINGULAR);
-    for (int x = threadIdx.x; x < kp * nM; x += blockDim.x)
-      M[(Dp + x % kp) + ldp * colp[x / kp]] = Pn[x];
-    // Z = A_dp U^{-1}: each dP row solved left to right, U from the staged rows; ZREG (levels of
-    // few parents, where this chain is the latency): a separator of at most 32 unknowns keeps
-    // the row in registers (one load and one store per entry, the same operations in the same
-    // order)
-    if (ZREG && kp <= 32) {
-      for (int a = threadIdx.x; a < ndP; a += blockDim.x) {
-        const size_t row = colp[a];
-        T z[32];
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (j < kp) z[j] = M[row + ldp * (Dp + j)];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          if (j < kp) {
-            T s = z[j];
-#pragma unroll
-            for (int i = 0; i < j; ++i) s -= z[i] * at(i, ndP + j);
-            z[j] = s * inv[j];
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (j < kp) M[row + ldp * (Dp + j)] = z[j];
-      }
-      return;
-    }
-    for (int a = threadIdx.x; a < ndP; a += blockDim.x) {
-      size_t row = colp[a];
-      for (int j = 0; j < kp; ++j) {
-        T s = M[row + ldp * (Dp + j)];
-        for (int i = 0; i < j; ++i) s -= M[row + ldp * (Dp + i)] * at(i, ndP + j);
-        M[row + ldp * (Dp + j)] = s * inv[j];
-      }
-    }
-    return;
-  }
   for (int j = 0; j < kp; ++j) {
     const int cj = Dp + j;
     if (threadIdx.x < 32) {
@@ -2090,56 +2080,199 @@ __global__ void __launch_bounds__(256) merge_panel_kernel(LevelDev d, int smem_b
   }
 }
 
-// Schur update of the parent's boundary block: M[dP, dP] -= Z W (64 x 64 tiles)
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.aligned;\n" ::: "memory"); }
+
+// W = L^{-1} P A_pd and Z = A_dp U^{-1} for the 32 boundary unknowns x0 .. x0 + 31 of a parent, from
+// the factored separator block A (kp <= 32 RS, in shared memory): four columns of W and four rows
+// of Z per warp, lanes over the separator's unknowns, one step per unknown.
+template <typename T, int RS>
+__device__ void panel_chunk(T* M, size_t ldp, int Dp, const int* tab, int x0, int ndP, int kp, const T* A, int lda,
+                            const int* q, const T* inv, T* Zt) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int CJ = 4;
+  const int ldz = kp | 1, nx = min(32, ndP - x0), w0 = CJ * warp;
+  for (int x = threadIdx.x; x < 32 * kp; x += blockDim.x) {
+    const int r = x & 31, j = x >> 5;
+    Zt[r * ldz + j] = M[tab[(size_t)(x0 + min(r, nx - 1)) * MERGE_TABW] + ldp * (Dp + j)];
+  }
+  T s[RS][CJ];
+  size_t pc[CJ];
+#pragma unroll
+  for (int c = 0; c < CJ; ++c) {
+    pc[c] = ldp * tab[(size_t)(x0 + min(w0 + c, nx - 1)) * MERGE_TABW];
+#pragma unroll
+    for (int t = 0; t < RS; ++t) {
+      const int i = min(lane + 32 * t, kp - 1);
+      s[t][c] = M[(Dp + q[i]) + pc[c]];
+    }
+  }
+  __syncthreads();                                 // Zt; every entry of W's columns is in registers
+  if (w0 < nx) {
+    for (int j = 0; j < kp; ++j) {
+      T x[CJ];
+#pragma unroll
+      for (int c = 0; c < CJ; ++c) x[c] = __shfl_sync(0xffffffffu, j < 32 ? s[0][c] : s[RS - 1][c], j & 31);
+#pragma unroll
+      for (int t = 0; t < RS; ++t) {
+        const int i = lane + 32 * t;
+        if (i > j && i < kp) {
+          const T l = A[i + lda * j];
+#pragma unroll
+          for (int c = 0; c < CJ; ++c) s[t][c] -= l * x[c];
+        }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < CJ; ++c)
+#pragma unroll
+      for (int t = 0; t < RS; ++t)
+        if (lane + 32 * t < kp && w0 + c < nx) M[(Dp + lane + 32 * t) + pc[c]] = s[t][c];
+    // Z: row z of z U = a, lanes over its entries
+#pragma unroll
+    for (int c = 0; c < CJ; ++c)
+#pragma unroll
+      for (int t = 0; t < RS; ++t) s[t][c] = Zt[(w0 + c) * ldz + min(lane + 32 * t, kp - 1)];
+    for (int j = 0; j < kp; ++j) {
+      T x[CJ];
+      const T iv = inv[j];
+#pragma unroll
+      for (int c = 0; c < CJ; ++c) x[c] = __shfl_sync(0xffffffffu, j < 32 ? s[0][c] : s[RS - 1][c], j & 31);
+#pragma unroll
+      for (int t = 0; t < RS; ++t) {
+        const int i = lane + 32 * t;
+        if (i > j && i < kp) {
+          const T g = A[j + lda * i] * iv;
+#pragma unroll
+          for (int c = 0; c < CJ; ++c) s[t][c] -= g * x[c];
+        }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < CJ; ++c)
+#pragma unroll
+      for (int t = 0; t < RS; ++t)
+        if (lane + 32 * t < kp) Zt[(w0 + c) * ldz + lane + 32 * t] = s[t][c] * inv[lane + 32 * t];
+  }
+  __syncthreads();
+  for (int x = threadIdx.x; x < 32 * kp; x += blockDim.x) {
+    const int r = x & 31, j = x >> 5;
+    if (r < nx) M[tab[(size_t)(x0 + r) * MERGE_TABW] + ldp * (Dp + j)] = Zt[r * ldz + j];
+  }
+  __syncthreads();
+}
+
+// The separator of each parent: LU of its block, W = L^{-1} P A_pd, Z = A_dp U^{-1}, and the block
+// replaced by [L~^{-1} \ U^{-1}] for the solve (kp <= INV_MAX).  gridDim.y CTAs (one cluster) share
+// a parent: each factors the block for itself (one barrier per pivot, fast_elim) and takes every
+// gridDim.y-th group of 32 boundary unknowns, so that on levels of few parents the columns and
+// rows spread over SMs; the first writes the inverse, after all have read the block.  What bounds
+// it: the kp steps of the three recurrences, about 0.1 us each in FP32 and 0.3 in FP64 (a FP64
+// instruction is 64 cycles; four columns share the one that scales U).
 template <typename T>
-__global__ void __launch_bounds__(256) merge_schur_kernel(LevelDev d) {
-  __shared__ T Zs[64][17];
-  __shared__ T Ws[16][65];
-  __shared__ int ra[64], cb[64];
+__global__ void __launch_bounds__(256) merge_panel_kernel(LevelDev d) {
+  extern __shared__ double pm_sm[];
+  __shared__ T inv[INV_MAX];
+  __shared__ int q[INV_MAX];
+  __shared__ int shi[8];
+  const int P = blockIdx.x;
+  const int ndP = d.pcount[2 * P], kp = d.pcount[2 * P + 1];
+  if (kp == 0) return;
+  const int* tab = d.ptab + (size_t)P * d.ldFp * TABW;
+  const size_t ldp = d.ldFp;
+  T* M = static_cast<T*>(d.Fp) + (size_t)P * ldp * ldp;
+  T* invg = static_cast<T*>(d.Pinv) + (size_t)P * d.sepcap;
+  int* pivg = d.ppiv + (size_t)P * d.sepcap;
+  const int Dp = d.gp.D();
+  if (kp > INV_MAX) {
+    if (blockIdx.y == 0) panel_large<T>(d, M, tab, ndP, kp, pivg, invg, shi);
+    return;
+  }
+  const int lda = kp | 1;
+  T* A = reinterpret_cast<T*>(pm_sm);
+  T* Zt = A + (size_t)kp * lda;
+  for (int x = threadIdx.x; x < kp * kp; x += blockDim.x) {
+    const int i = x % kp, j = x / kp;
+    A[i + lda * j] = M[(Dp + i) + ldp * (Dp + j)];
+  }
+  __syncthreads();
+  cluster_arrive();
+  const bool ok = kp <= 32 ? fast_elim<T, 8, 1>(A, lda, 0, kp, q, inv, shi, shi + 6)
+                           : fast_elim<T, 8, 2>(A, lda, 0, kp, q, inv, shi, shi + 6);
+  for (int x0 = 32 * blockIdx.y; x0 < ndP; x0 += 32 * gridDim.y) {
+    if (kp <= 32) panel_chunk<T, 1>(M, ldp, Dp, tab, x0, ndP, kp, A, lda, q, inv, Zt);
+    else panel_chunk<T, 2>(M, ldp, Dp, tab, x0, ndP, kp, A, lda, q, inv, Zt);
+  }
+  cluster_wait();
+  if (blockIdx.y != 0) return;
+  if (!ok && threadIdx.x == 0) atomicOr(d.err, ERR_SINGULAR);
+  if (kp <= 32) fast_invert<T, 8, 1>(A, lda, kp, inv, Zt);
+  else fast_invert<T, 8, 2>(A, lda, kp, inv, Zt);
+  for (int x = threadIdx.x; x < kp * kp; x += blockDim.x) M[(Dp + x % kp) + ldp * (Dp + x / kp)] = Zt[x];
+  for (int j = threadIdx.x; j < kp; j += blockDim.x) { invg[j] = inv[j]; pivg[j] = q[j]; }
+}
+
+// Schur update of the parent's boundary block: M[dP, dP] -= Z W, 32 x 32 tiles of two warps, each
+// thread 4 x 4.  In FP64 the multiply-adds bound it (64 cycles per warp instruction whatever its
+// lanes), so tiles are no larger than what pads a boundary of 60 - 100 unknowns little, a warp
+// whose 16 rows do not exist skips, and the sum runs over kp entries, not over a multiple of 16.
+template <typename T>
+__global__ void __launch_bounds__(64) merge_schur_kernel(LevelDev d) {
+  constexpr int TS = 32;
+  __shared__ T Zs[TS][17];
+  __shared__ T Ws[16][TS + 1];
+  __shared__ int ra[TS], cb[TS];
   const int P = blockIdx.z;
   const int ndP = d.pcount[2 * P], kp = d.pcount[2 * P + 1];
-  if (kp == 0 || ndP == 0) return;
-  const int tiles = (ndP + 63) / 64;
-  const int ti = blockIdx.x, tj = blockIdx.y;
-  if (ti >= tiles || tj >= tiles) return;
+  if (kp == 0) return;
+  const int tiles = (ndP + TS - 1) / TS;
   const int* tab = d.ptab + (size_t)P * d.ldFp * TABW;
   const size_t ldp = d.ldFp;
   T* M = static_cast<T*>(d.Fp) + (size_t)P * ldp * ldp;
   const int Dp = d.gp.D();
-  for (int x = threadIdx.x; x < 64; x += blockDim.x) {
-    int a = ti * 64 + x, b = tj * 64 + x;
-    ra[x] = a < ndP ? tab[(size_t)a * TABW] : -1;
-    cb[x] = b < ndP ? tab[(size_t)b * TABW] : -1;
-  }
-  __syncthreads();
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;   // 16 x 16 threads, 4 x 4 each
-  T acc[4][4] = {};
-  for (int j0 = 0; j0 < kp; j0 += 16) {
-    for (int x = threadIdx.x; x < 64 * 16; x += blockDim.x) {
-      int i = x % 64, j = x / 64;
-      Zs[i][j] = (ra[i] >= 0 && j0 + j < kp) ? M[ra[i] + ldp * (Dp + j0 + j)] : T(0);
-      int c = x % 64, jj = x / 64;
-      Ws[jj][c] = (cb[c] >= 0 && j0 + jj < kp) ? M[(Dp + j0 + jj) + ldp * cb[c]] : T(0);
-    }
-    __syncthreads();
+  const int tx = threadIdx.x % 8, ty = threadIdx.x / 8;   // 8 x 8 threads, 4 x 4 each
+  for (int ti = blockIdx.x; ti < tiles; ti += gridDim.x)
+    for (int tj = blockIdx.y; tj < tiles; tj += gridDim.y) {
+      __syncthreads();
+      {
+        const int x = threadIdx.x & 31, i = (threadIdx.x < 32 ? ti : tj) * TS + x;
+        (threadIdx.x < 32 ? ra : cb)[x] = i < ndP ? tab[(size_t)i * TABW] : -1;
+      }
+      __syncthreads();
+      const bool live = ti * TS + 16 * (threadIdx.x >> 5) < ndP;   // the warp's 16 rows
+      T acc[4][4] = {};
+      for (int j0 = 0; j0 < kp; j0 += 16) {
+        const int nj = min(16, kp - j0);
+        for (int x = threadIdx.x; x < TS * 16; x += 64) {
+          const int i = x % TS, j = x / TS;
+          Zs[i][j] = (ra[i] >= 0 && j < nj) ? M[ra[i] + ldp * (Dp + j0 + j)] : T(0);
+          const int jj = x % 16, c = x / 16;
+          Ws[jj][c] = (cb[c] >= 0 && jj < nj) ? M[(Dp + j0 + jj) + ldp * cb[c]] : T(0);
+        }
+        __syncthreads();
+        if (live) {
+#pragma unroll 4
+          for (int j = 0; j < nj; ++j) {
+            T z[4], w[4];
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      T z[4], w[4];
+            for (int u = 0; u < 4; ++u) { z[u] = Zs[ty * 4 + u][j]; w[u] = Ws[j][tx * 4 + u]; }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) { z[u] = Zs[ty * 4 + u][j]; w[u] = Ws[j][tx * 4 + u]; }
+            for (int u = 0; u < 4; ++u)
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+              for (int v = 0; v < 4; ++v) acc[u][v] += z[u] * w[v];
+          }
+        }
+        __syncthreads();
+      }
+      if (live) {
 #pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] += z[u] * w[v];
-    }
-    __syncthreads();
-  }
+        for (int v = 0; v < 4; ++v)
 #pragma unroll
-  for (int u = 0; u < 4; ++u)
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      int i = ty * 4 + u, c = tx * 4 + v;
-      if (ra[i] >= 0 && cb[c] >= 0) M[ra[i] + ldp * cb[c]] -= acc[u][v];
+          for (int u = 0; u < 4; ++u) {
+            const int i = ty * 4 + u, c = tx * 4 + v;
+            if (ra[i] >= 0 && cb[c] >= 0) M[ra[i] + ldp * cb[c]] -= acc[u][v];
+          }
+      }
     }
 }
 
@@ -2300,12 +2433,10 @@ __device__ __forceinline__ void upper_sweep(T* y, int ldy, int n, const T* LU, s
 }
 
 
-// Triangular blocks of order up to INV_MAX are inverted after the factorization (factor
-// kernels below), so that the solve applies them as one product per right-hand side instead of
-// a sequential sweep: [L\U] becomes [L~^{-1}\U^{-1}] with L~ the multipliers after all later
-// interchanges, and the pivot sequence becomes the permutation q, (P b)_i = b_{q_i}.
-constexpr int INV_MAX = 64;
-
+// Triangular blocks of order up to INV_MAX are inverted by the factorization, so that the solve
+// applies them as one product per right-hand side instead of a sequential sweep: [L\U] becomes
+// [L~^{-1}\U^{-1}] with L~ the multipliers after all later interchanges, and the pivot sequence
+// becomes the permutation q, (P b)_i = b_{q_i}.
 // v[:, c] = L~^{-1} v[q, c] (lower) or U^{-1} v[:, c] (upper) for c < nc, n <= INV_MAX, A the
 // inverted block (ld lda) in shared or global memory.  NT threads (the CTA), each holding at
 // most INV_MAX x 16 / NT outputs.
@@ -2340,45 +2471,6 @@ __device__ __forceinline__ void tri_apply(T* v, int ldv, int n, const T* A, size
   __syncthreads();
 }
 
-// In place on one GEPP block (n <= INV_MAX, column-major, ld lda; interchanges not applied to
-// earlier multipliers; rinv the reciprocal pivots): thread j moves column j's multipliers
-// through the later interchanges, then forms column j of L~^{-1} (below the diagonal) and of
-// U^{-1} (on and above it) from a shared-memory copy.  S and X: n * n each; q: n.
-template <typename T>
-__device__ void invert_lu_block(T* A, size_t lda, int n, const T* rinv, int* piv, T* S, T* X, int* q) {
-  for (int x = threadIdx.x; x < n * n; x += blockDim.x) S[x] = A[(x % n) + lda * (x / n)];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < n; ++i) q[i] = i;
-    for (int j = 0; j < n; ++j) { const int p = piv[j], t = q[j]; q[j] = q[p]; q[p] = t; }
-  }
-  for (int j = threadIdx.x; j < n; j += blockDim.x) {
-    T* sc = S + (size_t)n * j;
-    for (int t = j + 1; t < n; ++t) {
-      const int p = piv[t];
-      if (p != t) { const T a = sc[t]; sc[t] = sc[p]; sc[p] = a; }
-    }
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j < n; j += blockDim.x) {
-    T* xc = X + (size_t)n * j;
-    for (int i = j + 1; i < n; ++i) {          // L~ x = e_j (unit diagonal)
-      T s = S[i + (size_t)n * j];
-      for (int m = j + 1; m < i; ++m) s += S[i + (size_t)n * m] * xc[m];
-      xc[i] = -s;
-    }
-    xc[j] = rinv[j];                           // U x = e_j
-    for (int i = j - 1; i >= 0; --i) {
-      T s = T(0);
-      for (int m = i + 1; m <= j; ++m) s += S[i + (size_t)n * m] * xc[m];
-      xc[i] = -s * rinv[i];
-    }
-  }
-  __syncthreads();
-  for (int x = threadIdx.x; x < n * n; x += blockDim.x) A[(x % n) + lda * (x / n)] = X[x];
-  for (int i = threadIdx.x; i < n; i += blockDim.x) piv[i] = q[i];
-}
-
 template <typename T>
 __device__ __forceinline__ void gather_panel(T* dst, int nr, int ncl, const T* src, size_t ldsrc,
                                              const int* rowidx, size_t colbase) {
@@ -2388,42 +2480,6 @@ __device__ __forceinline__ void gather_panel(T* dst, int nr, int ncl, const T* s
     dst[x] = src[(size_t)rowidx[i] + ldsrc * (colbase + j)];
   }
 }
-
-// Inverse of each segment's remainder block (after the level's sparsification).
-template <typename T>
-__global__ void __launch_bounds__(64) seg_invert_kernel(LevelDev d) {
-  extern __shared__ double ism[];
-  const int sid = blockIdx.x;
-  const int e = d.cnt[sid], k = d.kk[sid], r = e - k;
-  if (r <= 0 || r > INV_MAX) return;
-  const size_t capS = d.capS;
-  T* S = reinterpret_cast<T*>(ism);
-  T* X = S + (size_t)r * r;
-  int* q = reinterpret_cast<int*>(X + (size_t)r * r);
-  T* Dg = static_cast<T*>(d.Dm) + (size_t)sid * capS * capS;
-  invert_lu_block<T>(Dg + k + capS * k, capS, r, static_cast<const T*>(d.Dinv) + (size_t)sid * capS,
-                     d.piv + (size_t)sid * capS, S, X, q);
-}
-
-// Inverse of each parent's separator block (after its elimination in the merge).
-template <typename T>
-__global__ void __launch_bounds__(64) sep_invert_kernel(LevelDev d) {
-  extern __shared__ double ism[];
-  const int P = blockIdx.x;
-  const int kp = d.pcount[2 * P + 1];
-  if (kp <= 0 || kp > INV_MAX) return;
-  const size_t ldp = d.ldFp;
-  const int Dp = d.gp.D();
-  T* S = reinterpret_cast<T*>(ism);
-  T* X = S + (size_t)kp * kp;
-  int* q = reinterpret_cast<int*>(X + (size_t)kp * kp);
-  T* M = static_cast<T*>(d.Fp) + (size_t)P * ldp * ldp;
-  invert_lu_block<T>(M + Dp + ldp * Dp, ldp, kp, static_cast<const T*>(d.Pinv) + (size_t)P * d.sepcap,
-                     d.ppiv + (size_t)P * d.sepcap, S, X, q);
-}
-
-template <typename T>
-size_t invert_smem() { return 2 * sizeof(T) * INV_MAX * INV_MAX + sizeof(int) * INV_MAX; }
 
 // The right-hand sides of a launch are split into gridDim.y groups (one CTA per group and
 // segment or separator: more CTAs where a level has few segments); this CTA's group becomes
@@ -2733,10 +2789,6 @@ static void sparsify_launch(const LevelDev& d, const LevelPlan& p, cudaStream_t 
                          cudaSharedmemCarveoutMaxShared);
     sparsify_kernel<T, NW><<<d.g.nseg(), NW * 32, smem, s>>>(d, smem);
   }
-  const int ism = (int)invert_smem<T>();
-  cudaFuncSetAttribute(seg_invert_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, ism);
-  note_launch();
-  seg_invert_kernel<T><<<d.g.nseg(), 64, ism, s>>>(d);
 }
 
 void launch_sparsify(const LevelDev& d, const LevelPlan& p, cudaStream_t s) {
@@ -2759,31 +2811,38 @@ static void merge_launch(const LevelDev& d, const LevelPlan& p, cudaStream_t s) 
     merge_assemble_kernel<T><<<grid, 256, 0, s>>>(d);
   }
   {
-    // shared memory for the staged separator rows: the geometric bound, at most 96 KB (larger
-    // parents take the global-memory path inside the kernel)
-    const size_t geo = (size_t)p.sepcap * p.ldFp * sizeof(T) + (size_t)p.ldFp * sizeof(int);
-    const int pm = (int)(geo < 96 * 1024 ? geo : 96 * 1024);
+    // the factored block and the larger of its inverse and the 32 boundary rows in work.  At most
+    // two parents per SM: a cluster of up to 8 CTAs per parent (more never helps: 256 boundary
+    // unknowns), else one
+    const size_t kb = (size_t)std::min(p.sepcap, INV_MAX), lda = kb | 1;
+    const int pm = (int)(sizeof(T) * (kb * lda + std::max(kb * kb, 32 * lda)));
+    cudaFuncSetAttribute(merge_panel_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, pm);
+    int cl = 1;
+    if (np <= 2 * sm_count())
+      while (cl < 8 && 32 * cl < p.ldFp) cl *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(np, cl);
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = pm;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1;
+    attr[0].val.clusterDim.y = cl;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
     note_launch();
-    if (np <= 2 * sm_count()) {      // at most two parents per SM: latency-bound, rows in registers
-      if (pm > 48 * 1024) cudaFuncSetAttribute(merge_panel_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, pm);
-      merge_panel_kernel<T, true><<<np, 256, pm, s>>>(d, pm);
-    } else {
-      if (pm > 48 * 1024) cudaFuncSetAttribute(merge_panel_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, pm);
-      merge_panel_kernel<T, false><<<np, 256, pm, s>>>(d, pm);
-    }
+    cudaLaunchKernelEx(&cfg, merge_panel_kernel<T>, d);
   }
-  {
-    const int ism = (int)invert_smem<T>();
-    cudaFuncSetAttribute(sep_invert_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, ism);
-    note_launch();
-    sep_invert_kernel<T><<<np, 64, ism, s>>>(d);
-  }
-  {
-    int tiles = (p.ldFp + 63) / 64;
-    dim3 grid(tiles, tiles, np);
-    note_launch();
-    if (d.schur_tc && d.fp32) merge_schur_tc_kernel<<<grid, 256, 0, s>>>(d);
-    else merge_schur_kernel<T><<<grid, 256, 0, s>>>(d);
+  note_launch();
+  if (d.schur_tc && d.fp32) {
+    const int tiles = (p.ldFp + 63) / 64;
+    merge_schur_tc_kernel<<<dim3(tiles, tiles, np), 256, 0, s>>>(d);
+  } else {
+    // tiles by the geometric bound (most are empty at the coarse levels), at most 32 x 32 of them
+    const int tiles = std::min((p.ldFp + 31) / 32, 32);
+    merge_schur_kernel<T><<<dim3(tiles, tiles, np), 64, 0, s>>>(d);
   }
   if (d.l > 1 && d.gp.nseg() > 0) {
     note_launch();
