@@ -2493,17 +2493,288 @@ __device__ __forceinline__ bool rhs_group(T*& X, int& nc, const VecLayout& lay) 
   return true;
 }
 
+// ---- level solves of segments and separators of at most INV_MAX unknowns.
+//
+// What bounds them: latency.  A level is two dependent launches per direction, each a chain of a
+// gather, two or three short products and a scatter.  So everything the factorization left is
+// staged before the wait on the preceding kernel, the products are three barriers apart, results
+// go from registers to the solve vector, and a thread holds one row and V right-hand sides (16
+// bytes): a multiply-add of the product costs 1/V loads of the matrix entry and one 16-byte load
+// of V vector entries instead of two loads each.
+template <typename T> struct RhsVec;
+template <> struct RhsVec<float> { static constexpr int V = 4; using type = float4; };
+template <> struct RhsVec<double> { static constexpr int V = 2; using type = double2; };
+__device__ __forceinline__ void axpy(float4& y, float a, const float4& x) {
+  y.x += a * x.x; y.y += a * x.y; y.z += a * x.z; y.w += a * x.w;
+}
+__device__ __forceinline__ void axpy(double2& y, double a, const double2& x) { y.x += a * x.x; y.y += a * x.y; }
+__device__ __forceinline__ float4 vzero(float) { return make_float4(0.f, 0.f, 0.f, 0.f); }
+__device__ __forceinline__ double2 vzero(double) { return make_double2(0.0, 0.0); }
+__device__ __forceinline__ float4 vsub(const float4& a, const float4& b) {
+  return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
+}
+__device__ __forceinline__ double2 vsub(const double2& a, const double2& b) { return make_double2(a.x - b.x, a.y - b.y); }
+
+// The CTA's right-hand sides: of the launch's nc (<= 16), groups of V, gridDim.y CTAs each taking
+// as many groups; lg = log2 of the groups rounded up to a power of two.  False: none left.
+template <typename T>
+__device__ __forceinline__ bool rhs_vec_group(T*& X, int& nc, int& lg, const VecLayout& lay) {
+  constexpr int V = RhsVec<T>::V;
+  const int tot = (nc + V - 1) / V, per = (tot + (int)gridDim.y - 1) / (int)gridDim.y, g0 = (int)blockIdx.y * per;
+  if (g0 >= tot) return false;
+  X += (size_t)(g0 * V) * (size_t)lay.cs;
+  nc = min(nc - g0 * V, per * V);
+  const int g = (nc + V - 1) / V;
+  lg = g > 4 ? 3 : g > 2 ? 2 : g > 1 ? 1 : 0;
+  return true;
+}
+
+// V right-hand sides of one node.  FP32: the chunked vector, whose 16 places per node always exist
+// (places past nc are carried along and never read out); FP64: columns, those past nc zero.
+__device__ __forceinline__ float4 rhs_load(const float* X, const VecLayout&, int node, int g, int) {
+  return reinterpret_cast<const float4*>(X + (size_t)node * 16)[g];
+}
+__device__ __forceinline__ double2 rhs_load(const double* X, const VecLayout& lay, int node, int g, int nc) {
+  double2 v;
+  v.x = 2 * g < nc ? X[lay.at(node, 2 * g)] : 0.0;
+  v.y = 2 * g + 1 < nc ? X[lay.at(node, 2 * g + 1)] : 0.0;
+  return v;
+}
+__device__ __forceinline__ void rhs_store(float* X, const VecLayout&, int node, int g, int, const float4& v) {
+  reinterpret_cast<float4*>(X + (size_t)node * 16)[g] = v;
+}
+__device__ __forceinline__ void rhs_store(double* X, const VecLayout& lay, int node, int g, int nc, const double2& v) {
+  if (2 * g < nc) X[lay.at(node, 2 * g)] = v.x;
+  if (2 * g + 1 < nc) X[lay.at(node, 2 * g + 1)] = v.y;
+}
+__device__ __forceinline__ void rhs_sub_atomic(float* X, const VecLayout&, int node, int g, int, const float4& v) {
+  atomicAdd(reinterpret_cast<float4*>(X + (size_t)node * 16) + g, make_float4(-v.x, -v.y, -v.z, -v.w));
+}
+__device__ __forceinline__ void rhs_sub_atomic(double* X, const VecLayout& lay, int node, int g, int nc, const double2& v) {
+  if (2 * g < nc) atomicAdd(X + lay.at(node, 2 * g), -v.x);
+  if (2 * g + 1 < nc) atomicAdd(X + lay.at(node, 2 * g + 1), -v.y);
+}
+
+// rows x (groups of right-hand sides): node rows into dst (pitch 16 values); FP32 reads a node's
+// groups with neighbouring threads, FP64 neighbouring rows of a column
+template <typename T, int NT, class Node>
+__device__ __forceinline__ void team_gather(const T* X, const VecLayout& lay, int nc, int lg, int n, Node node, T* dst) {
+  using Vt = typename RhsVec<T>::type;
+  const int tid = threadIdx.x, G = (nc + RhsVec<T>::V - 1) / RhsVec<T>::V;
+  if constexpr (sizeof(T) == 4) {
+    for (int x = tid; x < n << lg; x += NT) {
+      const int a = x >> lg, g = x & ((1 << lg) - 1);
+      if (g < G) reinterpret_cast<Vt*>(dst + 16 * a)[g] = rhs_load(X, lay, node(a), g, nc);
+    }
+  } else {
+    for (int g = tid >> 5; g < G; g += NT / 32)
+      for (int a = tid & 31; a < n; a += 32) reinterpret_cast<Vt*>(dst + 16 * a)[g] = rhs_load(X, lay, node(a), g, nc);
+  }
+}
+
+// for every row a < n and group g: acc = sum over j in [j0(a), j1(a)) of A[a + ld j] v[j][g], then out
+template <typename T, int NT, class J0, class J1, class Out>
+__device__ __forceinline__ void team_product(int n, int nc, int lg, const T* A, int ld, const T* v, J0 j0, J1 j1, Out out) {
+  using Vt = typename RhsVec<T>::type;
+  const int tid = threadIdx.x, G = (nc + RhsVec<T>::V - 1) / RhsVec<T>::V;
+  for (int x = tid; x < n << lg; x += NT) {
+    const int a = x >> lg, g = x & ((1 << lg) - 1);
+    if (g >= G) continue;
+    Vt acc = vzero(T(0));
+    const int je = j1(a);
+#pragma unroll 4
+    for (int j = j0(a); j < je; ++j) axpy(acc, A[a + ld * j], reinterpret_cast<const Vt*>(v + 16 * j)[g]);
+    out(a, g, acc);
+  }
+}
+
+// Shared memory of one segment of up to e unknowns: 2 panels of k r <= (e / 2)^2 values, the r x r
+// block, e rows of right-hand sides and r more, e nodes and r permutation entries
+__host__ __device__ inline size_t seg_team_bytes(int e, int tb) {
+  const size_t pc = (size_t)(e / 2 + 1) * (e / 2 + 1);
+  return ((2 * pc + (size_t)e * e + 32 * (size_t)e) * tb + 8 * (size_t)e + 15) / 16 * 16;
+}
+// ... of one separator of up to kp unknowns with up to nd boundary unknowns: the kp x nd panel (odd
+// pitch), the kp x kp block, kp rows of right-hand sides twice, nd rows (backward; and 256 partial
+// vectors), kp + 2 nd table entries and kp permutation entries
+__host__ __device__ inline size_t sep_team_bytes(int kp, int nd, int tb) {
+  return ((size_t)(kp | 1) * nd + (size_t)kp * kp + 32 * (size_t)kp + 16 * (size_t)nd) * tb + 256 * 16 + 4 * (2 * (size_t)kp + 2 * (size_t)nd) + 64;
+}
+
+// Forward, per segment: b_r -= T^T b_s; y_r = L^{-1} P b_r; b_s -= Z y_r.
+// Backward, per segment: x_r = U^{-1} (y_r - W x_s); x_s -= T x_r.
+template <typename T, int NT>
+__global__ void __launch_bounds__(NT) seg_team_kernel(LevelDev d, SolveCaps cap, T* X, int nc, VecLayout lay, int bwd) {
+  pdl_trigger();
+  extern __shared__ float4 tsm4[];
+  const int sid = blockIdx.x, tid = threadIdx.x;
+  int lg = 0;
+  const bool some = rhs_vec_group(X, nc, lg, lay);
+  const int e = some ? d.cnt[sid] : 0, k = some ? d.kk[sid] : 0;
+  int r = e - k;
+  if (e > cap.vrows) { if (tid == 0) atomicOr(d.err, ERR_CAPACITY); r = 0; }
+  if (r == 0) { pdl_wait(); return; }
+  const int capS = d.capS;
+  T* S = reinterpret_cast<T*>(tsm4);                     // skeleton rows, then remainder rows, pitch 16
+  T* R = S + 16 * k;
+  T* Yb = S + 16 * e;                                    // the new remainder rows
+  T* Ts = Yb + 16 * r;                                   // forward: T^T, rows permuted (r x k); backward: T (k x r)
+  T* Ps = Ts + k * r;                                    // forward: Z (k x r); backward: W (r x k)
+  T* LU = Ps + k * r;                                    // r x r
+  int* nds = reinterpret_cast<int*>(LU + r * r);
+  int* q = nds + e;
+  const int* snodes = d.snodes + (size_t)sid * capS;     // nodes in [skeleton | remainder] order
+  const int* piv = d.piv + (size_t)sid * capS;
+  const T* Tm = static_cast<const T*>(d.T) + (size_t)sid * capS * capS;
+  const T* Dg = static_cast<const T*>(d.Dm) + (size_t)sid * capS * capS;
+  const int lane = tid & 31, w = tid >> 5;
+  constexpr int NWT = NT / 32;
+  for (int a = tid; a < e; a += NT) nds[a] = snodes[a];
+  for (int a = tid; a < r; a += NT) q[a] = piv[a];
+  __syncthreads();
+  for (int j = w; j < r; j += NWT) {
+    for (int i = lane; i < r; i += 32) LU[i + r * j] = Dg[(k + i) + (size_t)capS * (k + j)];
+    if (!bwd) {
+      const int jq = q[j];
+      for (int i = lane; i < k; i += 32) {
+        Ts[j + r * i] = Tm[i + (size_t)capS * jq];
+        Ps[i + k * j] = Dg[i + (size_t)capS * (k + j)];
+      }
+    } else {
+      for (int i = lane; i < k; i += 32) Ts[i + k * j] = Tm[i + (size_t)capS * j];
+    }
+  }
+  if (bwd)
+    for (int j = w; j < k; j += NWT)
+      for (int i = lane; i < r; i += 32) Ps[i + r * j] = Dg[(k + i) + (size_t)capS * j];
+  pdl_wait();
+  using Vt = typename RhsVec<T>::type;
+  team_gather<T, NT>(X, lay, nc, lg, e, [&](int a) { return nds[(a < k || bwd) ? a : k + q[a - k]]; }, S);
+  __syncthreads();
+  auto zero = [](int) { return 0; };
+  // remainder rows less their skeleton part (forward in pivot order)
+  team_product<T, NT>(r, nc, lg, bwd ? Ps : Ts, r, S, zero, [&](int) { return k; }, [&](int a, int g, const Vt& acc) {
+    Vt* v = reinterpret_cast<Vt*>(R + 16 * a) + g;
+    *v = vsub(*v, acc);
+  });
+  __syncthreads();
+  // the inverted triangle (forward: unit lower, diagonal not stored)
+  team_product<T, NT>(r, nc, lg, LU, r, R, [&](int a) { return bwd ? a : 0; }, [&](int a) { return bwd ? r : a; },
+                      [&](int a, int g, Vt acc) {
+                        if (!bwd) axpy(acc, T(1), reinterpret_cast<const Vt*>(R + 16 * a)[g]);
+                        reinterpret_cast<Vt*>(Yb + 16 * a)[g] = acc;
+                        rhs_store(X, lay, nds[k + a], g, nc, acc);
+                      });
+  if (k == 0) return;
+  __syncthreads();
+  // skeleton rows less their remainder part
+  team_product<T, NT>(k, nc, lg, bwd ? Ts : Ps, k, Yb, zero, [&](int) { return r; }, [&](int a, int g, const Vt& acc) {
+    rhs_store(X, lay, nds[a], g, nc, vsub(reinterpret_cast<const Vt*>(S + 16 * a)[g], acc));
+  });
+}
+
+// Separator of each parent: forward y_p = L^{-1} P b_p, then b_dP -= Z y_p added atomically
+// (a boundary unknown is shared by up to four parents; the order of their contributions is
+// not fixed; FP32: four right-hand sides per atomic); backward x_p = U^{-1} (y_p - W x_dP), the sum
+// over the boundary split over the threads that kp rows leave idle.
+template <typename T, int NT>
+__global__ void __launch_bounds__(NT) sep_team_kernel(LevelDev d, SolveCaps cap, T* X, int nc, VecLayout lay, int bwd) {
+  pdl_trigger();
+  extern __shared__ float4 tsm4[];
+  using Vt = typename RhsVec<T>::type;
+  const int P = blockIdx.x, tid = threadIdx.x;
+  int lg = 0;
+  const bool some = rhs_vec_group(X, nc, lg, lay);
+  const int ndP = d.pcount[2 * P];
+  int kp = some ? d.pcount[2 * P + 1] : 0;
+  if (kp > cap.yrows || ndP > cap.drows) { if (tid == 0) atomicOr(d.err, ERR_CAPACITY); kp = 0; }
+  if (kp == 0) { pdl_wait(); return; }
+  const int* tab = d.ptab + (size_t)P * d.ldFp * TABW;
+  const size_t ldp = d.ldFp;
+  const T* M = static_cast<const T*>(d.Fp) + (size_t)P * ldp * ldp;
+  const int Dp = d.gp.D();
+  const int* piv = d.ppiv + (size_t)P * d.sepcap;
+  Vt* part = reinterpret_cast<Vt*>(tsm4);                // 256 partial vectors (backward)
+  T* y = reinterpret_cast<T*>(part + 256);               // kp rows, pitch 16
+  T* y2 = y + 16 * kp;
+  T* xd = y2 + 16 * kp;                                  // ndP rows (backward)
+  T* LU = xd + 16 * ndP;                                 // kp x kp
+  const int ldw = kp | 1;
+  T* Pn = LU + kp * kp;                                  // forward: Z (ndP x kp); backward: W (kp x ndP, pitch ldw)
+  int* pos = reinterpret_cast<int*>(Pn + (size_t)ldw * ndP);
+  int* node = pos + ndP;                                 // boundary, then separator
+  int* q = node + ndP + kp;
+  for (int x = tid; x < ndP + kp; x += NT) {
+    if (x < ndP) pos[x] = tab[(size_t)x * TABW];
+    node[x] = tab[(size_t)x * TABW + 7];
+  }
+  for (int a = tid; a < kp; a += NT) q[a] = piv[a];
+  __syncthreads();
+  const int lane = tid & 31, w = tid >> 5;
+  constexpr int NWT = NT / 32;
+  for (int j = w; j < kp; j += NWT) {
+    for (int i = lane; i < kp; i += 32) LU[i + kp * j] = M[(Dp + i) + ldp * (Dp + j)];
+    if (!bwd)
+      for (int i = lane; i < ndP; i += 32) Pn[i + ndP * j] = M[pos[i] + ldp * (Dp + j)];
+  }
+  if (bwd)
+    for (int b = w; b < ndP; b += NWT)
+      for (int i = lane; i < kp; i += 32) Pn[i + ldw * b] = M[(Dp + i) + ldp * pos[b]];
+  pdl_wait();
+  team_gather<T, NT>(X, lay, nc, lg, kp, [&](int a) { return node[ndP + (bwd ? a : q[a])]; }, y);
+  if (bwd) team_gather<T, NT>(X, lay, nc, lg, ndP, [&](int b) { return node[b]; }, xd);
+  __syncthreads();
+  auto zero = [](int) { return 0; };
+  if (!bwd) {
+    team_product<T, NT>(kp, nc, lg, LU, kp, y, zero, [](int a) { return a; }, [&](int a, int g, Vt acc) {
+      axpy(acc, T(1), reinterpret_cast<const Vt*>(y + 16 * a)[g]);
+      reinterpret_cast<Vt*>(y2 + 16 * a)[g] = acc;
+      rhs_store(X, lay, node[ndP + a], g, nc, acc);
+    });
+    __syncthreads();
+    team_product<T, NT>(ndP, nc, lg, Pn, ndP, y2, zero, [&](int) { return kp; }, [&](int b, int g, const Vt& acc) {
+      rhs_sub_atomic(X, lay, node[b], g, nc, acc);
+    });
+  } else {
+    // y_p - W x_dP: (kp rows x groups) outputs, each summed by 2^ls threads
+    const int G = (nc + RhsVec<T>::V - 1) / RhsVec<T>::V, n = kp << lg;
+    int ls = 0;
+    while (ls < 4 && (n << (ls + 1)) <= NT) ++ls;
+    for (int x0 = 0; x0 < n << ls; x0 += NT) {
+      const int x = x0 + tid, o = x >> ls, s = x & ((1 << ls) - 1), a = o >> lg, g = o & ((1 << lg) - 1);
+      Vt acc = vzero(T(0));
+      if (a < kp && g < G) {
+#pragma unroll 4
+        for (int b = s; b < ndP; b += 1 << ls) axpy(acc, Pn[a + ldw * b], reinterpret_cast<const Vt*>(xd + 16 * b)[g]);
+      }
+      part[tid] = acc;
+      __syncwarp();
+      if (s == 0 && a < kp && g < G) {
+        Vt t = reinterpret_cast<const Vt*>(y + 16 * a)[g];
+        for (int i = 0; i < 1 << ls; ++i) t = vsub(t, part[tid + i]);
+        reinterpret_cast<Vt*>(y + 16 * a)[g] = t;
+      }
+      __syncwarp();
+    }
+    __syncthreads();
+    team_product<T, NT>(kp, nc, lg, LU, kp, y, [](int a) { return a; }, [&](int) { return kp; }, [&](int a, int g, const Vt& acc) {
+      rhs_store(X, lay, node[ndP + a], g, nc, acc);
+    });
+  }
+}
+
+// The same for levels with larger segments or separators.
 // Forward, per segment: b_r -= T^T b_s; y_r = L^{-1} P b_r; b_s -= Z y_r.
 // Backward, per segment: x_r = U^{-1} (y_r - W x_s); x_s -= T x_r.
 template <typename T, int NT>
 __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 16) seg_solve_kernel(LevelDev d, SolveCaps cap, T* X, int nc, VecLayout lay, int bwd) {
   pdl_trigger();
   extern __shared__ double smd[];
-  if (!rhs_group(X, nc, lay)) return;
+  if (!rhs_group(X, nc, lay)) { pdl_wait(); return; }
   const int sid = blockIdx.x;
   const int e = d.cnt[sid], k = d.kk[sid], r = e - k;
-  if (r == 0 || e == 0) return;
-  if (e > cap.vrows) { if (threadIdx.x == 0) atomicOr(d.err, ERR_CAPACITY); return; }
+  if (r == 0 || e == 0) { pdl_wait(); return; }
+  if (e > cap.vrows) { if (threadIdx.x == 0) atomicOr(d.err, ERR_CAPACITY); pdl_wait(); return; }
   const int capS = d.capS;
   T* v = reinterpret_cast<T*>(smd);                      // e x SC, [skeleton | remainder]
   T* LUsm = v + (size_t)cap.vrows * SC;                  // r x r LU (when r <= lucap)
@@ -2597,11 +2868,11 @@ template <typename T, int NT>
 __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 16) sep_solve_kernel(LevelDev d, SolveCaps cap, T* X, int nc, VecLayout lay, int bwd) {
   pdl_trigger();
   extern __shared__ double smd[];
-  if (!rhs_group(X, nc, lay)) return;
+  if (!rhs_group(X, nc, lay)) { pdl_wait(); return; }
   const int P = blockIdx.x;
   const int ndP = d.pcount[2 * P], kp = d.pcount[2 * P + 1];
-  if (kp == 0) return;
-  if (kp > cap.yrows) { if (threadIdx.x == 0) atomicOr(d.err, ERR_CAPACITY); return; }
+  if (kp == 0) { pdl_wait(); return; }
+  if (kp > cap.yrows) { if (threadIdx.x == 0) atomicOr(d.err, ERR_CAPACITY); pdl_wait(); return; }
   const int* tab = d.ptab + (size_t)P * d.ldFp * TABW;
   const size_t ldp = d.ldFp;
   const T* M = static_cast<const T*>(d.Fp) + (size_t)P * ldp * ldp;
@@ -2887,44 +3158,66 @@ bool level_solve_caps(const LevelDev& d, const int* lmax, SolveCaps* out) {
   // CTA widths before any tuning: 2-warp segment CTAs where segments have at most 32 unknowns
   sc.seg_nt = d.capS <= 32 ? 64 : 256;
   sc.sep_nt = 256;
+  // FP64: right-hand sides over more CTAs on levels of few segments or separators (1799 -> 1617 us
+  // of level solves at 1023^2 with 16: a CTA's FP64 pipe is the limit there); FP32 stays on one
+  // (336 against 343 us)
   sc.seg_split = sc.sep_split = 1;
+  if (!d.fp32) {
+    while (sc.seg_split < 8 && 2 * sc.seg_split * d.g.nseg() <= sm_count()) sc.seg_split *= 2;
+    while (sc.sep_split < 8 && 2 * sc.sep_split * d.gp.nbox() <= sm_count()) sc.sep_split *= 2;
+  }
   sc.sep_smem = (size_t)(sep_fixed + TB * mx((long long)sc.lucap * sc.lucap, sc.qcap));
+  // the forms for at most INV_MAX unknowns, where all of a segment or separator fits
+  sc.seg_team = lmax[0] <= INV_MAX;
+  sc.sep_team = lmax[1] <= INV_MAX && lmax[2] <= DCAP &&
+                sep_team_bytes(sc.yrows, (int)lmax[2], (int)TB) <= (size_t)budget;
+  if (sc.sep_team) sc.drows = (int)lmax[2];
+  if (sc.seg_team) {
+    // measured (level solves of one solve): FP32 1023^2 with 16 right-hand sides 324 us with two
+    // warps per segment, 423 with eight; FP64 1632 and 1542
+    sc.seg_nt = d.fp32 ? 64 : 256;
+    sc.seg_smem = seg_team_bytes(sc.vrows, (int)TB);
+  }
+  if (sc.sep_team) sc.sep_smem = sep_team_bytes(sc.yrows, sc.drows, (int)TB);
   *out = sc;
   return true;
 }
 
 template <typename T>
 static void level_solve(const LevelDev& d, const SolveCaps& sc, T* X, int nrhs, VecLayout lay, int bwd, cudaStream_t s) {
-  cudaFuncSetAttribute(seg_solve_kernel<T, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sc.seg_smem);
-  cudaFuncSetAttribute(seg_solve_kernel<T, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sc.seg_smem);
-  cudaFuncSetAttribute(sep_solve_kernel<T, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sc.sep_smem);
-  cudaFuncSetAttribute(sep_solve_kernel<T, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sc.sep_smem);
   for (int c0 = 0; c0 < nrhs; c0 += SC) {
     const int nc = nrhs - c0 < SC ? nrhs - c0 : SC;
     T* Xc = X + (size_t)(c0 / SC) * lay.chunk;
-    auto seg_go = [&](int dir) {
+    auto go = [&](auto kern, int n, int split, int threads, size_t smem) {
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       note_launch();
-      const dim3 grid(d.g.nseg(), sc.seg_split < nc ? sc.seg_split : nc);
-      if (sc.seg_nt == 64)  // 2-warp CTAs: four times as many resident per SM
-        launch_pdl(seg_solve_kernel<T, 64>, grid, dim3(64), sc.seg_smem, s, d, sc, Xc, nc, lay, dir);
-      else
-        launch_pdl(seg_solve_kernel<T, 256>, grid, dim3(256), sc.seg_smem, s, d, sc, Xc, nc, lay, dir);
+      launch_pdl(kern, dim3(n, split < nc ? split : nc), dim3(threads), smem, s, d, sc, Xc, nc, lay, bwd);
     };
-    auto sep_go = [&](int dir) {
-      note_launch();
-      const dim3 grid(d.gp.nbox(), sc.sep_split < nc ? sc.sep_split : nc);
-      if (sc.sep_nt == 64)
-        launch_pdl(sep_solve_kernel<T, 64>, grid, dim3(64), sc.sep_smem, s, d, sc, Xc, nc, lay, dir);
-      else
-        launch_pdl(sep_solve_kernel<T, 256>, grid, dim3(256), sc.sep_smem, s, d, sc, Xc, nc, lay, dir);
+    auto seg_go = [&]() {
+      const int n = d.g.nseg();
+      if (n == 0) return;
+      if (sc.seg_team) {
+        if (sc.seg_nt == 64) go(seg_team_kernel<T, 64>, n, sc.seg_split, 64, sc.seg_smem);
+        else go(seg_team_kernel<T, 256>, n, sc.seg_split, 256, sc.seg_smem);
+      } else if (sc.seg_nt == 64) {       // 2-warp CTAs: four times as many resident per SM
+        go(seg_solve_kernel<T, 64>, n, sc.seg_split, 64, sc.seg_smem);
+      } else {
+        go(seg_solve_kernel<T, 256>, n, sc.seg_split, 256, sc.seg_smem);
+      }
     };
-    if (!bwd) {
-      if (d.g.nseg() > 0) seg_go(0);
-      sep_go(0);
-    } else {
-      sep_go(1);
-      if (d.g.nseg() > 0) seg_go(1);
-    }
+    auto sep_go = [&]() {
+      const int n = d.gp.nbox();
+      if (sc.sep_team) {
+        if (sc.sep_nt == 64) go(sep_team_kernel<T, 64>, n, sc.sep_split, 64, sc.sep_smem);
+        else go(sep_team_kernel<T, 256>, n, sc.sep_split, 256, sc.sep_smem);
+      } else if (sc.sep_nt == 64) {
+        go(sep_solve_kernel<T, 64>, n, sc.sep_split, 64, sc.sep_smem);
+      } else {
+        go(sep_solve_kernel<T, 256>, n, sc.sep_split, 256, sc.sep_smem);
+      }
+    };
+    if (!bwd) { seg_go(); sep_go(); }
+    else { sep_go(); seg_go(); }
   }
 }
 

@@ -192,6 +192,8 @@ struct SolveCaps {
   int yrows;     // separator: skeleton rows of the right-hand-side block (>= every kp)
   size_t seg_smem, sep_smem;
   int seg_nt, sep_nt;   // CTA widths of the segment / separator solve kernels (64 or 256)
+  int seg_team, sep_team;   // 1: no segment / separator of the level exceeds INV_MAX unknowns and
+                        // everything of one fits in shared memory
   int seg_split, sep_split;   // right-hand-side groups per segment / separator (CTAs along y)
 };
 
