@@ -837,6 +837,7 @@ spalu_status spalu_factor_create(spalu_nd_t nd, const spalu_opts* o, spalu_facto
       d.near_radius = o->near_radius; d.h0 = o->h0; d.seed = o->seed;
       d.schur_tc = (o->schur_tc && f32) ? 1 : 0;
       d.sketch_tc = (o->sketch_tc && f32) ? 1 : 0;
+      sparsify_wide_plan(p, &d);
       d.L = L;
       d.pred_mode = PRED_OFF; d.pred_margin = 0.35; d.pred = nullptr;
       d.log10eps = o->eps_id > 0.0 ? std::log10(o->eps_id) : -16.0;

@@ -25,6 +25,8 @@
 #include <cfloat>
 #include <cmath>
 
+#include <cooperative_groups.h>
+
 #include "pred_infer.cuh"
 #include "spalu_internal.h"
 #include "work.cuh"
@@ -1414,6 +1416,13 @@ __global__ void __launch_bounds__(1024) seg_order_kernel(const int* cnt, int nse
   for (int s = threadIdx.x; s < nseg; s += blockDim.x) order[atomicAdd(&start[key(cnt[s])], 1)] = s;
 }
 
+constexpr int WIDE_EMAX = 512;
+// Segments of at most 32 unknowns go to a cluster from this many entries of B; larger ones always do.
+// Measured per level, one CTA / cluster: e 31 with 4000 entries 291 / 322 us, e 31 with 9000 312 / 291,
+// e 46 with 4500 457 / 406, e 267 without neighbours (the last separator) 12.9 ms / 0.74 ms.
+constexpr int WIDE_MIN = 5000;
+__device__ __forceinline__ bool wide_takes(const LevelDev& d, const SegCtx& S, int tb);   // below
+
 // Shared memory of a segment besides its blocks (norms, permutations, pivots, reciprocals), and the
 // values of its interpolation matrix (k (e - k) <= e^2 / 4, and room for the 8 probe rows)
 __host__ __device__ inline size_t sparsify_smem_small(int e, int tbytes) {
@@ -1435,11 +1444,15 @@ __global__ void __launch_bounds__(NWT * 32, NWT == NW ? 4 : 16) sparsify_kernel(
   __syncthreads();
   const int e = S.e;
   const int capS = d.capS;
+  // Beside a wide kernel this one starts early: what follows both waits for both through the last CTA,
+  // which ends no sooner than the clusters do (with no such launch before it the wait is none)
+  auto leave = [&]() { if (blockIdx.x == gridDim.x - 1) pdl_wait(); };
+  if (wide_takes(d, S, sizeof(T))) return leave();     // sparsify_wide_kernel's
   int* perm_out = d.perm + (size_t)sid * capS;
   if (threadIdx.x == 0) atomicMax(d.lstat + LS_EMAX, e);
   if (e == 0) {
     if (threadIdx.x == 0) { d.kk[sid] = 0; d.hs[sid] = 0; }
-    return;
+    return leave();
   }
   const size_t ld = d.ldF;
   const T* F1 = static_cast<const T*>(d.F) + (size_t)S.b1 * ld * ld;
@@ -1818,6 +1831,778 @@ __global__ void __launch_bounds__(NWT * 32, NWT == NW ? 4 : 16) sparsify_kernel(
     atomicAdd(d.flops, work_done);
     atomicAdd(d.flops + 2, (unsigned long long)((k * r + e * e) * sizeof(T) + 2 * e * sizeof(int)));
   }
+  leave();
+}
+
+// W = L^{-1} P A_pd and Z = A_dp U^{-1} for the 32 boundary unknowns x0 .. x0 + 31 of a parent, from
+// the factored block A (kp <= 32 RS, in shared memory), posn(x) the place of unknown x in M: four columns of W and four rows
+// of Z per warp, lanes over the separator's unknowns, one step per unknown.
+template <typename T, int RS, class Pos>
+__device__ void panel_chunk(T* M, size_t ldp, int Dp, Pos posn, int x0, int ndP, int kp, const T* A, int lda,
+                            const int* q, const T* inv, T* Zt) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int CJ = 4;
+  const int ldz = kp | 1, nx = min(32, ndP - x0), w0 = CJ * warp;
+  for (int x = threadIdx.x; x < 32 * kp; x += blockDim.x) {
+    const int r = x & 31, j = x >> 5;
+    Zt[r * ldz + j] = M[posn(x0 + min(r, nx - 1)) + ldp * (Dp + j)];
+  }
+  T s[RS][CJ];
+  size_t pc[CJ];
+#pragma unroll
+  for (int c = 0; c < CJ; ++c) {
+    pc[c] = ldp * posn(x0 + min(w0 + c, nx - 1));
+#pragma unroll
+    for (int t = 0; t < RS; ++t) {
+      const int i = min(lane + 32 * t, kp - 1);
+      s[t][c] = M[(Dp + q[i]) + pc[c]];
+    }
+  }
+  __syncthreads();                                 // Zt; every entry of W's columns is in registers
+  if (w0 < nx) {
+    for (int j = 0; j < kp; ++j) {
+      T x[CJ];
+#pragma unroll
+      for (int c = 0; c < CJ; ++c) {
+        T v = s[0][c];
+#pragma unroll
+        for (int t = 1; t < RS; ++t) v = (j >> 5) == t ? s[t][c] : v;
+        x[c] = __shfl_sync(0xffffffffu, v, j & 31);
+      }
+#pragma unroll
+      for (int t = 0; t < RS; ++t) {
+        const int i = lane + 32 * t;
+        if (i > j && i < kp) {
+          const T l = A[min(i, kp - 1) + lda * j];
+#pragma unroll
+          for (int c = 0; c < CJ; ++c) s[t][c] -= l * x[c];
+        }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < CJ; ++c)
+#pragma unroll
+      for (int t = 0; t < RS; ++t)
+        if (lane + 32 * t < kp && w0 + c < nx) M[(Dp + lane + 32 * t) + pc[c]] = s[t][c];
+    // Z: row z of z U = a, lanes over its entries
+#pragma unroll
+    for (int c = 0; c < CJ; ++c)
+#pragma unroll
+      for (int t = 0; t < RS; ++t) s[t][c] = Zt[(w0 + c) * ldz + min(lane + 32 * t, kp - 1)];
+    for (int j = 0; j < kp; ++j) {
+      T x[CJ];
+      const T iv = inv[j];
+#pragma unroll
+      for (int c = 0; c < CJ; ++c) {
+        T v = s[0][c];
+#pragma unroll
+        for (int t = 1; t < RS; ++t) v = (j >> 5) == t ? s[t][c] : v;
+        x[c] = __shfl_sync(0xffffffffu, v, j & 31);
+      }
+#pragma unroll
+      for (int t = 0; t < RS; ++t) {
+        const int i = lane + 32 * t;
+        if (i > j && i < kp) {
+          const T g = A[j + lda * min(i, kp - 1)] * iv;
+#pragma unroll
+          for (int c = 0; c < CJ; ++c) s[t][c] -= g * x[c];
+        }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < CJ; ++c)
+#pragma unroll
+      for (int t = 0; t < RS; ++t)
+        if (lane + 32 * t < kp) Zt[(w0 + c) * ldz + lane + 32 * t] = s[t][c] * inv[min(lane + 32 * t, kp - 1)];
+  }
+  __syncthreads();
+  for (int x = threadIdx.x; x < 32 * kp; x += blockDim.x) {
+    const int r = x & 31, j = x >> 5;
+    if (r < nx) M[posn(x0 + r) + ldp * (Dp + j)] = Zt[r * ldz + j];
+  }
+  __syncthreads();
+}
+
+// ------------------------------------------------------------ sparsify: one cluster per segment
+// On levels of few segments one CTA per segment leaves most SMs idle, and in FP64 the sketch, the
+// QR and the dense products of a segment are bound by one SM's FP64 pipe (2 multiply-adds per
+// clock).  Here a cluster of C CTAs shares a segment:
+//   - rows of the sketch (whole Philox groups of four) are dealt out, each CTA forms and keeps its
+//     own (the same sums as in sketch_far);
+//   - QR with the rows where they are (row i of the pivot order is local row i / C of CTA i mod C;
+//     missing rows are zero): per step every CTA sends its partial products with the pivot column,
+//     and one its row i, to all, and after one cluster barrier all take the same decisions from the
+//     same numbers, so nothing has to be sent back;
+//   - interpolation, transforms and elimination by columns or elements over all CTAs, on the
+//     segment's place in global memory, cluster barriers between.
+// What bounds it: the pivots' serial chain (a cluster barrier, two block reductions, a FP64 square
+// root and a quotient each) and the FP64 pipe of C SMs.  One CTA / cluster, 1023 x 1023 at eps 1e-8:
+// Helmholtz, 10 segments of up to 155 unknowns, 33.2 / 3.6 ms; 24 of up to 101, 10.2 / 1.7 ms;
+// diffusion, 24 of up to 57, 858 / 535 us.
+// Columns: warp w of NSW = min(8, ceil(e / 32)) column sets x RG row groups holds set w mod NSW (and
+// set w + 8 where e > 256), rows r mod RG = w / NSW; the warps of row group 0 own the columns' state.
+namespace cg = cooperative_groups;
+
+struct WideShape {             // sizes that every CTA of the cluster derives alike
+  int C, rank, e, NS, NSW, RG, EC;
+};
+
+__host__ __device__ inline int wide_rows(int C, int nN, int far_rows, bool whole) {
+  const int nr = (nN + C - 1) / C;
+  return whole ? nr + (far_rows + C - 1) / C : nr + 4 * (((far_rows + 3) / 4 + C - 1) / C);
+}
+// Shared memory of a segment of e unknowns with nb neighbours, a sketch chunk of four far unknowns
+// at least: exchange buffers (two parities of C sums and a row per column), partial sums of the row
+// groups, coefficients, reciprocals, permutation and pivots, neighbour table; then the rows and the
+// chunk, whose place the elimination of up to INV_MAX remainders takes later
+__host__ __device__ inline size_t wide_bytes(int e, int nb, int C, int halves, int h0, int p_over, int tb) {
+  const size_t ec = (size_t)(e + 31) / 32 * 32;
+  const size_t fixed = (2 * (C + 1) * ec + ec + (ec > 256 ? ec : 256)) * 8 + (size_t)e * tb + 8 * (size_t)e + 9 * (size_t)nb + 64;
+  const int hcap = h0 > 2 * (e + p_over) ? h0 : 2 * (e + p_over);
+  const size_t m = wide_rows(C, halves * NEAR_MAX, hcap, false) | 1;
+  const size_t y = m * e + 4 * (size_t)halves * (e + m), lu = 2 * INV_MAX * (INV_MAX + 1);
+  return fixed + (y > lu ? y : lu) * tb;
+}
+// whether the segment is the wide kernel's (asked by both kernels)
+__device__ __forceinline__ bool wide_takes(const LevelDev& d, const SegCtx& S, int tb) {
+  const int halves = d.symmetric ? 1 : 2;
+  return d.wide > 1 && S.e <= WIDE_EMAX && (S.e > 32 || halves * S.e * S.nb >= WIDE_MIN) &&
+         wide_bytes(S.e, S.nb, d.wide, halves, d.h0, d.p_over, tb) <= (size_t)d.wide_smem;
+}
+
+// The QR above; every thread of every CTA calls it.  Yl: mloc rows (pitch ldl) of e columns.  R rows
+// go to Rg (global, leading dimension ldr, columns in place) from CTA 0; perm in every CTA.
+template <typename T, int MS>
+__device__ int wide_qr(cg::cluster_group& cl, const WideShape& W, T* Yl, int ldl, int mloc, int m, double eps, int kstop,
+                       double* xch, double* part, T* coef, int* perm, T* Rg, size_t ldr, double* sc, unsigned* red) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int e = W.e, C = W.C, rank = W.rank, EC = W.EC;
+  const int kmax = min(min(m, e), kstop);
+  const int set0 = warp % W.NSW, rg = warp / W.NSW;
+  const bool on = rg < W.RG, own = on && rg == 0;
+  int col[MS], pos[MS];
+  bool val[MS];
+  T* yc[MS];
+  double n1[MS], g2[MS];
+  const double tol3z = sqrt(DBL_EPSILON);
+  const double tie = (1.0 - TIE_RTOL) * (1.0 - TIE_RTOL);
+#pragma unroll
+  for (int t = 0; t < MS; ++t) {
+    col[t] = 32 * (set0 + 8 * t) + lane;
+    val[t] = on && col[t] < e;
+    yc[t] = Yl + ldl * min(col[t], e - 1);
+    pos[t] = val[t] ? col[t] : e;
+    n1[t] = g2[t] = 0.0;
+  }
+  int par = 0;
+  // sums over the row groups and the CTAs of one value per column; in v[] for the owners
+  auto gather_sum = [&](double (&v)[MS], const T* row) {
+#pragma unroll
+    for (int t = 0; t < MS; ++t)
+      if (val[t]) part[rg * EC + col[t]] = v[t];
+    __syncthreads();
+    double* buf = xch + (size_t)par * (C + 1) * EC;          // C x EC sums, then the row
+    if (own) {
+#pragma unroll
+      for (int t = 0; t < MS; ++t)
+        if (val[t]) {
+          double q = part[col[t]];
+          for (int g = 1; g < W.RG; ++g) q += part[g * EC + col[t]];
+          for (int c = 0; c < C; ++c) {
+            double* pb = cl.map_shared_rank(buf, c);
+            pb[rank * EC + col[t]] = q;
+            if (row) pb[C * EC + col[t]] = (double)row[ldl * col[t]];
+          }
+        }
+    }
+    cl.sync();
+    if (own) {
+#pragma unroll
+      for (int t = 0; t < MS; ++t)
+        if (val[t]) {
+          double q[8];
+#pragma unroll
+          for (int c = 0; c < 8; ++c) q[c] = c < C ? buf[min(c, C - 1) * EC + col[t]] : 0.0;
+#pragma unroll
+          for (int o = 4; o > 0; o >>= 1)
+            if (o < C)
+#pragma unroll
+              for (int c = 0; c < 4; ++c)
+                if (c < o) q[c] += q[c + o];
+          v[t] = q[0];
+        }
+    }
+    par ^= 1;
+    return buf + C * EC;
+  };
+  // pivot among the positions >= i: key = position * 65536 + column, the same in every thread
+  auto choose = [&](int i) {
+    unsigned hi = 0, lo = 0;
+#pragma unroll
+    for (int t = 0; t < MS; ++t)
+      if (own && pos[t] >= i && pos[t] < e) hi = max(hi, bits_hi(n1[t]));
+    hi = __reduce_max_sync(0xffffffffu, hi);
+#pragma unroll
+    for (int t = 0; t < MS; ++t)
+      if (own && pos[t] >= i && pos[t] < e && bits_hi(n1[t]) == hi) lo = max(lo, bits_lo(n1[t]));
+    lo = __reduce_max_sync(0xffffffffu, lo);
+    if (lane == 0) { red[2 * warp] = hi; red[2 * warp + 1] = lo; }
+    __syncthreads();
+    unsigned long long mx = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) mx = max(mx, ((unsigned long long)red[2 * q] << 32) | red[2 * q + 1]);
+    const long long thr = dbits(__longlong_as_double((long long)mx) * tie);
+    unsigned best = 0xffffffffu, first = 0xffffffffu;
+#pragma unroll
+    for (int t = 0; t < MS; ++t)
+      if (own && pos[t] >= i && pos[t] < e) {
+        const unsigned key = ((unsigned)pos[t] << 16) | (unsigned)col[t];
+        first = min(first, key);
+        if (dbits(n1[t]) >= thr) best = min(best, key);
+      }
+    best = __reduce_min_sync(0xffffffffu, best);
+    first = __reduce_min_sync(0xffffffffu, first);
+    if (lane == 0) { red[16 + warp] = best; red[24 + warp] = first; }
+    __syncthreads();
+    best = first = 0xffffffffu;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) { best = min(best, red[16 + q]); first = min(first, red[24 + q]); }
+    return best != 0xffffffffu ? best : first;               // first: only where a norm is not a number
+  };
+  double v[MS];
+#pragma unroll
+  for (int t = 0; t < MS; ++t) {
+    T a = T(0);
+    if (val[t])
+      for (int r = rg; r < mloc; r += W.RG) { const T y = yc[t][r]; a += y * y; }
+    v[t] = (double)a;
+  }
+  gather_sum(v, nullptr);
+#pragma unroll
+  for (int t = 0; t < MS; ++t) { n1[t] = v[t]; g2[t] = tol3z * v[t]; }
+  unsigned key = choose(0);
+  int k = kmax;
+  for (int i = 0; i < kmax; ++i) {
+    const int p = (int)(key & 0xffffu), pp = (int)(key >> 16);
+#pragma unroll
+    for (int t = 0; t < MS; ++t) {
+      if (val[t] && col[t] == p) pos[t] = i;
+      else if (val[t] && pos[t] == i) pos[t] = pp;
+    }
+    // local rows of the pivot order from i on: q C + rank >= i
+    const int l0 = i > rank ? (i - rank + C - 1) / C : 0;
+    const int lr0 = l0 + ((rg - l0) % W.RG + W.RG) % W.RG;
+    const T* x = Yl + ldl * p;
+#pragma unroll
+    for (int t = 0; t < MS; ++t) {
+      T a = T(0);
+      if (val[t] && pos[t] >= i)
+#pragma unroll 4
+        for (int r = lr0; r < mloc; r += W.RG) a += x[r] * yc[t][r];
+      v[t] = (double)a;
+    }
+    const double* yrow = gather_sum(v, rank == i % C ? Yl + i / C : nullptr);
+#pragma unroll
+    for (int t = 0; t < MS; ++t)
+      if (own && val[t] && col[t] == p) { sc[0] = v[t]; sc[1] = yrow[p]; }
+    __syncthreads();
+    if (warp == 0) {
+      const T s = (T)sc[0], x0 = (T)sc[1];
+      const T normx = qr_norm(s);
+      int stop = 0;
+      double re = sc[6];
+      if (i == 0) {
+        re = eps * (double)normx;
+        if (normx == T(0)) stop = 2;
+      }
+      if (!stop && ((double)normx <= re || normx == T(0))) stop = 1;
+      const T alpha = x0 >= T(0) ? -normx : normx;
+      const T den = s + (x0 >= T(0) ? x0 : -x0) * normx;
+      const T c2 = den > T(0) ? T(1) / den : T(0);
+      __syncwarp();
+      if (lane == 0) {
+        sc[2] = (double)alpha;
+        sc[3] = (double)(x0 - alpha);
+        sc[4] = (double)c2;
+        sc[5] = (double)stop;
+        if (i == 0) sc[6] = re;
+      }
+    }
+    __syncthreads();
+    const int stop = (int)sc[5];
+    if (stop) { k = stop == 2 ? 0 : i; break; }
+    bool low = false;
+    {
+      const T alpha = (T)sc[2], v0 = (T)sc[3], c2 = (T)sc[4];
+#pragma unroll
+      for (int t = 0; t < MS; ++t)
+        if (own && val[t]) {
+          const bool act = pos[t] > i;
+          const T yi = (T)yrow[col[t]];
+          const T cj = act ? c2 * ((T)v[t] - alpha * yi) : T(0);
+          const T rij = yi - cj * v0;
+          coef[col[t]] = cj;
+          if (act) {
+            if (rank == 0) Rg[i + ldr * col[t]] = rij;
+            if (dbits(n1[t]) != 0) {
+              const double rd = (double)rij, sn = n1[t] - rd * rd;
+              const long long sb = dbits(sn) < 0 ? 0 : dbits(sn);
+              if (sb <= dbits(g2[t])) low = true;
+              else n1[t] = __longlong_as_double(sb);
+            }
+          } else if (col[t] == p && rank == 0) {
+            Rg[i + ldr * col[t]] = alpha;
+          }
+        }
+    }
+    low = __syncthreads_or(low);
+    if (i + 1 >= kmax) break;
+    const int l1 = i + 1 > rank ? (i + 1 - rank + C - 1) / C : 0;
+    const int lr1 = l1 + ((rg - l1) % W.RG + W.RG) % W.RG;
+    const T* vc = Yl + ldl * p;
+#pragma unroll
+    for (int t = 0; t < MS; ++t) {
+      double a2 = 0.0;
+      if (val[t] && pos[t] > i) {
+        const T cj = coef[col[t]];
+#pragma unroll 4
+        for (int r = lr1; r < mloc; r += W.RG) {
+          const T y = yc[t][r] - cj * vc[r];
+          yc[t][r] = y;
+          if (low) a2 += (double)y * (double)y;
+        }
+      }
+      v[t] = a2;
+    }
+    if (low) {
+      gather_sum(v, nullptr);
+#pragma unroll
+      for (int t = 0; t < MS; ++t)
+        if (own && val[t] && pos[t] > i) { n1[t] = v[t]; g2[t] = tol3z * v[t]; }
+    }
+    key = choose(i + 1);       // its barriers also order the update before the next products
+  }
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < MS; ++t)
+    if (own && val[t]) perm[pos[t]] = col[t];
+  cl.sync();                   // perm; R in global memory; no CTA still reads another's buffers
+  return k;
+}
+
+// T = R_1^{-1} R_2 over the cluster's warps: two columns per warp, lanes over the rows, R in global
+// memory (column of position b at ldr perm[b]) and, where it fits, R_1 in pool; rinv: k values in
+// every CTA.
+template <typename T>
+__device__ void wide_interp(const WideShape& W, const T* Rg, size_t ldr, int k, const int* perm, T* Tg, size_t ldt, T* rinv,
+                            T* pool, size_t room) {
+  const int lane = threadIdx.x & 31, e = W.e;
+  const bool staged = (size_t)k * k <= room;         // addresses stay below k^2 and k: loads may run ahead
+  if (staged)
+    for (int b = threadIdx.x >> 5; b < k; b += 8)
+      for (int a = lane; a <= b; a += 32) pool[a + k * b] = Rg[a + ldr * perm[b]];
+  constexpr int CJ = 2, MK = WIDE_EMAX / 32;
+  for (int a = threadIdx.x; a < k; a += blockDim.x) rinv[a] = T(1) / Rg[a + ldr * perm[a]];
+  __syncthreads();
+  const int nk = (k + 31) / 32;
+  for (int j0 = CJ * ((threadIdx.x >> 5) * W.C + W.rank); j0 < e - k; j0 += CJ * 8 * W.C) {
+    T s[MK][CJ];
+#pragma unroll
+    for (int t = 0; t < MK; ++t)
+#pragma unroll
+      for (int q = 0; q < CJ; ++q) {
+        s[t][q] = T(0);
+        if (t < nk && lane + 32 * t < k) s[t][q] = Rg[min(lane + 32 * t, k - 1) + ldr * perm[min(k + j0 + q, e - 1)]];
+      }
+#pragma unroll
+    for (int tb = MK - 1; tb >= 0; --tb) {
+      if (tb >= nk) continue;
+      for (int a = min(32 * tb + 31, k - 1); a >= 32 * tb; --a) {
+        const T* ra = staged ? pool + k * a : Rg + ldr * perm[a];
+        const T iv = rinv[a];
+        T x[CJ];
+#pragma unroll
+        for (int q = 0; q < CJ; ++q) x[q] = __shfl_sync(0xffffffffu, s[tb][q], a & 31);
+#pragma unroll
+        for (int t = 0; t <= tb; ++t) {
+          const int b = lane + 32 * t;
+          if (b < a) {
+            const T g = ra[min(b, k - 1)] * iv;
+#pragma unroll
+            for (int q = 0; q < CJ; ++q) s[t][q] -= g * x[q];
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < MK; ++t)
+#pragma unroll
+      for (int q = 0; q < CJ; ++q)
+        if (t < nk && lane + 32 * t < k && j0 + q < e - k)
+          Tg[lane + 32 * t + ldt * (j0 + q)] = s[t][q] * rinv[min(lane + 32 * t, k - 1)];
+  }
+}
+
+// LU with partial pivoting of the n x n block A (global memory, leading dimension lda) by the
+// cluster, columns dealt out (column c to CTA c mod C) and held in shared memory: the owner of the
+// next pivot column updates it first, finds its pivot and sends the multipliers to all.  Multipliers
+// are not interchanged afterwards.  cs: n ceil(n / C) values; mb: 2 (n + 2) doubles.
+template <typename T>
+__device__ bool wide_lu(cg::cluster_group& cl, const WideShape& W, T* A, size_t lda, int n, int* piv, T* inv, T* cs, double* mb) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, C = W.C, rank = W.rank;
+  const int mine = (n - rank + C - 1) / C;
+  for (int x = threadIdx.x; x < mine * n; x += blockDim.x) cs[x] = A[x % n + lda * (rank + C * (x / n))];
+  cl.sync();                   // cs; every CTA runs, so that its buffers may be written
+  bool ok = true;
+  // warp 0 of the owner: pivot of column j, multipliers and pivot row to every CTA
+  auto prepare = [&](int j) {
+    T* c = cs + (size_t)n * (j / C);
+    unsigned hi = 0, lo = 0, best = 0xffffffffu;
+    for (int r = j + lane; r < n; r += 32) hi = max(hi, abs_hi(c[r]));
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    for (int r = j + lane; r < n; r += 32)
+      if (abs_hi(c[r]) == hi) lo = max(lo, abs_lo(c[r]));
+    lo = __reduce_max_sync(0xffffffffu, lo);
+    for (int r = j + lane; r < n; r += 32)
+      if (abs_hi(c[r]) == hi && abs_lo(c[r]) == lo) best = min(best, (unsigned)r);
+    best = __reduce_min_sync(0xffffffffu, best);
+    const int p = (int)min(best, (unsigned)(n - 1));
+    const T pv = c[p], old = c[j];
+    const T iv = (hi | lo) ? T(1) / pv : T(0);
+    __syncwarp();
+    if (lane == 0) { c[p] = old; c[j] = pv; }
+    __syncwarp();
+    double* b = mb + (size_t)(j & 1) * (n + 2);
+    for (int r = j + 1 + lane; r < n; r += 32) {
+      const T l = c[r] * iv;
+      c[r] = l;
+      for (int q = 0; q < C; ++q) cl.map_shared_rank(b, q)[r] = (double)l;
+    }
+    if (lane < C) {
+      double* pb = cl.map_shared_rank(b, lane);
+      pb[n] = (double)p;
+      pb[n + 1] = (double)iv;
+    }
+  };
+  if (rank == 0 && warp == 0) prepare(0);
+  cl.sync();
+  for (int j = 0; j < n; ++j) {
+    const double* b = mb + (size_t)(j & 1) * (n + 2);
+    const int p = (int)b[n];
+    const T iv = (T)b[n + 1];
+    if (iv == T(0)) ok = false;
+    if (rank == 0 && threadIdx.x == 0) { piv[j] = p; inv[j] = iv; }
+    auto column = [&](int c) {
+      T* y = cs + (size_t)n * (c / C);
+      const T u = y[p], o = y[j];
+      __syncwarp();
+      for (int r = j + 1 + lane; r < n; r += 32) y[r] = (r == p ? o : y[r]) - (T)b[r] * u;
+      __syncwarp();
+      if (lane == 0) y[j] = u;
+      __syncwarp();
+    };
+    // the CTA's columns above j, the next pivot column by warp 0 first
+    const bool mynext = j + 1 < n && (j + 1) % C == rank;
+    const int c0 = j + 1 + ((rank - (j + 1)) % C + C) % C;     // first own column above j
+    if (mynext) {
+      if (warp == 0) { column(j + 1); prepare(j + 1); }
+      else
+        for (int c = c0 + C * warp; c < n; c += 7 * C) column(c);
+    } else {
+      for (int c = c0 + C * warp; c < n; c += 8 * C) column(c);
+    }
+    cl.sync();
+  }
+  for (int x = threadIdx.x; x < mine * n; x += blockDim.x) A[x % n + lda * (rank + C * (x / n))] = cs[x];
+  return ok;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) sparsify_wide_kernel(LevelDev d) {
+  extern __shared__ double sm[];
+  __shared__ SegCtx S;
+  __shared__ int nearlist[NEAR_MAX];
+  __shared__ int nnear_sh, nfar_sh, okf;
+  __shared__ double sc[8];
+  __shared__ unsigned red[32];
+  __shared__ int shi[8];
+  pdl_trigger();               // sparsify_kernel, on this level's other segments
+  cg::cluster_group cl = cg::this_cluster();
+  WideShape W;
+  W.C = d.wide;
+  W.rank = (int)cl.block_rank();
+  const int sid = blockIdx.x / d.wide;
+  if (threadIdx.x == 0) seg_context(d, sid, S);
+  __syncthreads();
+  const int e = S.e, capS = d.capS, rank = W.rank, C = W.C;
+  if (!wide_takes(d, S, sizeof(T))) return;          // the whole cluster: sparsify_kernel's
+  const bool lead = rank == 0 && threadIdx.x == 0;
+  if (lead) atomicMax(d.lstat + LS_EMAX, e);
+  if (e == 0) {
+    if (lead) { d.kk[sid] = 0; d.hs[sid] = 0; }
+    return;
+  }
+  W.e = e;
+  W.NS = (e + 31) / 32;
+  W.NSW = min(8, W.NS);
+  W.RG = 8 / W.NSW;
+  W.EC = 32 * W.NS;
+  const size_t ld = d.ldF;
+  const T* F1 = static_cast<const T*>(d.F) + (size_t)S.b1 * ld * ld;
+  const T* F2 = static_cast<const T*>(d.F) + (size_t)S.b2 * ld * ld;
+  T* Dg = static_cast<T*>(d.Dm) + (size_t)sid * capS * capS;
+  T* Tg = static_cast<T*>(d.T) + (size_t)sid * capS * capS;
+  T* Ykeep = static_cast<T*>(d.Yg) + (size_t)sid * d.Ycap * capS;
+  const int halves = d.symmetric ? 1 : 2;
+  // shared memory
+  char* q = reinterpret_cast<char*>(sm);
+  double* xch = reinterpret_cast<double*>(q); q += (size_t)2 * (C + 1) * W.EC * 8;
+  double* part = reinterpret_cast<double*>(q); q += (size_t)max(256, W.EC) * 8;
+  T* coef = reinterpret_cast<T*>(q); q += (size_t)W.EC * 8;
+  T* rinv = reinterpret_cast<T*>(q); q += (size_t)e * sizeof(T);
+  int* perm = reinterpret_cast<int*>(q); q += (size_t)e * 4;
+  int* piv = reinterpret_cast<int*>(q); q += (size_t)e * 4;
+  int* tb_node = reinterpret_cast<int*>(q); q += (size_t)S.nb * 4;
+  short* tb_p1 = reinterpret_cast<short*>(q); q += (size_t)S.nb * 2;
+  short* tb_p2 = reinterpret_cast<short*>(q); q += (size_t)S.nb * 2;
+  unsigned char* tb_nf = reinterpret_cast<unsigned char*>(q); q += S.nb;
+  q = reinterpret_cast<char*>(((uintptr_t)q + 15) & ~(uintptr_t)15);
+  T* pool = reinterpret_cast<T*>(q);
+  const size_t room = ((size_t)d.wide_smem - (size_t)(q - reinterpret_cast<char*>(sm))) / sizeof(T);
+  const NbrTab tb{tb_node, tb_p1, tb_p2, tb_nf, true};
+  {
+    const NbrTab none{nullptr, nullptr, nullptr, nullptr, false};
+    for (int f = threadIdx.x; f < S.nb; f += blockDim.x) {
+      const Nbr n = nbr_get(d, S, none, f);
+      tb_node[f] = n.node;
+      tb_p1[f] = (short)n.p1;
+      tb_p2[f] = (short)n.p2;
+      tb_nf[f] = n.nearf ? 1 : 0;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const int lane = threadIdx.x;
+    int nn = 0;
+    for (int base = 0; base < S.nb; base += 32) {
+      const bool isnear = base + lane < S.nb && tb_nf[min(base + lane, S.nb - 1)] != 0;
+      const unsigned msk = __ballot_sync(0xffffffffu, isnear);
+      const int at = nn + __popc(msk & ((1u << lane) - 1u));
+      if (isnear && at < NEAR_MAX) nearlist[at] = base + lane;
+      nn += __popc(msk);
+    }
+    if (lane == 0) {
+      if (nn > NEAR_MAX) atomicOr(d.err, ERR_CAPACITY);
+      nnear_sh = min(nn, NEAR_MAX);
+      nfar_sh = S.nb - nn;
+    }
+  }
+  cl.sync();                   // the lists; every CTA runs, so that its buffers may be written
+  const int nnear = nnear_sh, nN = halves * nnear, nF = halves * nfar_sh;
+  const int hcap = max(d.h0, 2 * (e + d.p_over)), hmax = min(nF, hcap);
+  const bool small = e + d.p_over <= 2 * d.h0;
+  int h = min((nF <= d.h0) ? nF : small ? min(hmax, 2 * d.h0) : min(hmax, d.h0), hmax);
+  const int nrl = (nN + C - 1) / C;
+  auto bget = [&](int t, int f, int c) { return bval_q<T>(d, S, F1, F2, nbr_get(d, S, tb, f), t, c); };
+  int k = 0, passes = 0, have = 0;
+  unsigned long long work_done = 0;
+  while (true) {
+    const bool full = h >= nF;
+    const int hh = full ? nF : h, m = nN + hh;
+    const int mloc = wide_rows(C, nN, hh, full), ldl = mloc | 1;
+    T* Yl = pool;
+    if (lead && !full) work_done += work::sketch(hh, nF, e);
+    for (int x = threadIdx.x; x < ldl * e; x += blockDim.x) Yl[x] = T(0);
+    __syncthreads();
+    for (int x = threadIdx.x; x < nrl * e; x += blockDim.x) {
+      const int a = rank + C * (x % nrl), c = x / nrl;
+      if (a < nN) Yl[x % nrl + ldl * c] = bget(a / nnear, nearlist[a % nnear], c);
+    }
+    if (full) {
+      // Phi = I: far row t nfar + j, j the place of the far neighbour among the far ones
+      for (int f = threadIdx.x; f < S.nb; f += blockDim.x) {
+        int before = 0;
+        bool isnear = false;
+        for (int a = 0; a < nnear; ++a) {
+          if (nearlist[a] < f) ++before;
+          if (nearlist[a] == f) isnear = true;
+        }
+        if (isnear) continue;
+        for (int t = 0; t < halves; ++t) {
+          const int j = t * nfar_sh + f - before;
+          if (j % C == rank)
+            for (int c = 0; c < e; ++c) Yl[nrl + j / C + ldl * c] = bget(t, f, c);
+        }
+      }
+    } else {
+      // this CTA's groups of four rows: g = rank + C gl; those below `have` were kept
+      const int ng = (hh + 3) / 4, ngl = ng > rank ? (ng - rank + C - 1) / C : 0;
+      const int kept = have / 4 > rank ? (have / 4 - rank + C - 1) / C : 0, gn = ngl - kept, nr = 4 * gn;
+      T* Yr = Yl + nrl + 4 * kept;
+      if (gn > 0) {
+        const size_t left = room - (size_t)ldl * e;
+        const int ch = (int)min((size_t)SK_CHUNK_MAX, left / ((size_t)halves * (e + nr))) & ~(SK_CHUNK - 1);
+        const int cw = ch > 0 ? ch : (int)max((size_t)1, min((size_t)SK_CHUNK, left / ((size_t)halves * (e + nr))));
+        T* Bc = Yl + (size_t)ldl * e;
+        T* Gc = Bc + (size_t)halves * cw * e;
+        for (int f0 = 0; f0 < S.nb; f0 += cw) {
+          const int nc = min(cw, S.nb - f0), rows = halves * nc;
+          for (int x = threadIdx.x; x < nc * e; x += blockDim.x) {
+            Bc[x % nc + (size_t)rows * (x / nc)] = bget(0, f0 + x % nc, x / nc);
+            if (halves == 2) Bc[nc + x / e + (size_t)rows * (x % e)] = bget(1, f0 + x / e, x % e);
+          }
+          for (int x = threadIdx.x; x < gn * rows; x += blockDim.x) {
+            const int gi = x % gn, row = x / gn, t = row / nc, f = f0 + row % nc;
+            float z[4] = {0.f, 0.f, 0.f, 0.f};
+            if (!tb_nf[f]) sketch_gauss4(d.seed, d.l, sid, rank + C * (kept + gi), tb_node[f], t, z);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) Gc[4 * gi + i + (size_t)nr * row] = (T)z[i];
+          }
+          __syncthreads();
+          for (int x = threadIdx.x; x < nr * e; x += blockDim.x) {
+            const int rr = x % nr, c = x / nr;
+            const T* g = Gc + rr;
+            const T* bc = Bc + (size_t)rows * c;
+            T y = Yr[rr + ldl * c];
+            for (int b0 = 0; b0 < nc; b0 += SK_CHUNK) {
+              const int b1 = min(nc, b0 + SK_CHUNK);
+              T acc = T(0);
+#pragma unroll 4
+              for (int row = b0; row < b1; ++row) acc += g[(size_t)nr * row] * bc[row];
+              if (halves == 2) {
+#pragma unroll 4
+                for (int row = nc + b0; row < nc + b1; ++row) acc += g[(size_t)nr * row] * bc[row];
+              }
+              y += acc;
+            }
+            Yr[rr + ldl * c] = y;
+          }
+          __syncthreads();
+        }
+      }
+      // scale; rows past hh are zero; rows that a larger sketch would continue are kept
+      const T scl = (T)(1.0 / sqrt((double)hh));
+      const bool keep = e > hh - d.p_over;
+      for (int x = threadIdx.x; x < 4 * ngl * e; x += blockDim.x) {
+        const int lr = x % (4 * ngl), c = x / (4 * ngl), rr = 4 * (rank + C * (lr / 4)) + lr % 4;
+        T* y = Yl + nrl + lr + ldl * c;
+        T val = lr < 4 * kept ? Ykeep[rr + (size_t)d.Ycap * c] : *y;
+        if (rr >= hh) val = T(0);
+        if (keep && lr >= 4 * kept && rr < hh) Ykeep[rr + (size_t)d.Ycap * c] = val;
+        *y = val * scl;
+      }
+      if (keep) have = hh & ~3;
+    }
+    __syncthreads();
+    const int kstop = (!full && h < nF) ? max(1, hh - d.p_over + 1) : e;
+    k = 0;
+    if (m > 0) {
+      k = e <= 256 ? wide_qr<T, 1>(cl, W, Yl, ldl, mloc, m, d.eps, kstop, xch, part, coef, perm, Dg, capS, sc, red)
+                   : wide_qr<T, 2>(cl, W, Yl, ldl, mloc, m, d.eps, kstop, xch, part, coef, perm, Dg, capS, sc, red);
+    } else {
+      for (int j = threadIdx.x; j < e; j += blockDim.x) perm[j] = j;
+      __syncthreads();
+    }
+    ++passes;
+    if (lead) work_done += work::qr(m, e, k);
+    if (!full && k > h - d.p_over && h < nF) {
+      h = min(2 * h, hmax);
+      continue;
+    }
+    break;
+  }
+  const int r = e - k;
+  if (k > 0) wide_interp<T>(W, Dg, capS, k, perm, Tg, capS, rinv, pool, room);
+  cl.sync();                                          // R is read, T is written
+  // ---- transformed diagonal block, in its place in global memory
+  const int gt = rank * blockDim.x + threadIdx.x, gs = C * blockDim.x;
+  for (int x = gt; x < e * e; x += gs) {
+    const int a = x % e, b = x / e, pa = perm[a], pb = perm[b];
+    Dg[a + (size_t)capS * b] = F1[(S.s1 + pa) + ld * (S.s1 + pb)] + F2[(S.s2 + pa) + ld * (S.s2 + pb)];
+  }
+  cl.sync();
+  if (k > 0 && r > 0) {
+    for (int x = gt; x < e * r; x += gs) {
+      const int a = x % e, b = x / e;
+      T s = T(0);
+#pragma unroll 4
+      for (int c = 0; c < k; ++c) s += Dg[a + (size_t)capS * c] * Tg[c + (size_t)capS * b];
+      Dg[a + (size_t)capS * (k + b)] -= s;
+    }
+    cl.sync();
+    for (int x = gt; x < r * e; x += gs) {
+      const int a = x % r, b = x / r;
+      T s = T(0);
+#pragma unroll 4
+      for (int c = 0; c < k; ++c) s += Tg[c + (size_t)capS * a] * Dg[c + (size_t)capS * b];
+      Dg[(k + a) + (size_t)capS * b] -= s;
+    }
+    cl.sync();
+  }
+  // ---- remainder
+  bool ok = true;
+  if (r > 0 && r <= INV_MAX) {
+    const int lda = r | 1;
+    T* A = pool;
+    T* Zt = A + (size_t)r * lda;
+    for (int x = threadIdx.x; x < r * r; x += blockDim.x) A[x % r + lda * (x / r)] = Dg[(k + x % r) + (size_t)capS * (k + x / r)];
+    __syncthreads();
+    ok = r <= 32 ? fast_elim<T, 8, 1>(A, lda, 0, r, piv, rinv, shi, &okf) : fast_elim<T, 8, 2>(A, lda, 0, r, piv, rinv, shi, &okf);
+    auto posn = [](int x) { return x; };
+    for (int x0 = 32 * rank; x0 < k; x0 += 32 * C) {
+      if (r <= 32) panel_chunk<T, 1>(Dg, capS, k, posn, x0, k, r, A, lda, piv, rinv, Zt);
+      else panel_chunk<T, 2>(Dg, capS, k, posn, x0, k, r, A, lda, piv, rinv, Zt);
+    }
+    cl.sync();
+    for (int x = gt; x < k * k; x += gs) {
+      const int a = x % k, b = x / k;
+      T s = T(0);
+#pragma unroll 4
+      for (int j = 0; j < r; ++j) s += Dg[a + (size_t)capS * (k + j)] * Dg[(k + j) + (size_t)capS * b];
+      Dg[a + (size_t)capS * b] -= s;
+    }
+    if (rank == 0) {
+      if (r <= 32) fast_invert<T, 8, 1>(A, lda, r, rinv, Zt);
+      else fast_invert<T, 8, 2>(A, lda, r, rinv, Zt);
+      for (int x = threadIdx.x; x < r * r; x += blockDim.x) Dg[(k + x % r) + (size_t)capS * (k + x / r)] = Zt[x];
+    }
+  } else if (r > INV_MAX && k == 0) {
+    ok = wide_lu<T>(cl, W, Dg, capS, r, piv, rinv, pool, xch);
+  } else if (r > INV_MAX && rank == 0) {
+    ok = block_gepp<T>(Dg, capS, k, r, e, piv, rinv, shi, false);
+    for (int a = threadIdx.x; a < k; a += blockDim.x)
+      for (int j = 0; j < r; ++j) {
+        T s = Dg[a + (size_t)capS * (k + j)];
+        for (int i2 = 0; i2 < j; ++i2) s -= Dg[a + (size_t)capS * (k + i2)] * Dg[(k + i2) + (size_t)capS * (k + j)];
+        Dg[a + (size_t)capS * (k + j)] = s * rinv[j];
+      }
+    __syncthreads();
+    for (int x = threadIdx.x; x < k * k; x += blockDim.x) {
+      const int a = x % k, b = x / k;
+      T s = T(0);
+      for (int j = 0; j < r; ++j) s += Dg[a + (size_t)capS * (k + j)] * Dg[(k + j) + (size_t)capS * b];
+      Dg[a + (size_t)capS * b] -= s;
+    }
+  }
+  __syncthreads();
+  if (rank != 0) return;
+  if (!ok && threadIdx.x == 0) atomicOr(d.err, ERR_SINGULAR);
+  for (int j = threadIdx.x; j < e; j += blockDim.x) {
+    d.perm[(size_t)sid * capS + j] = perm[j];
+    d.snodes[(size_t)sid * capS + j] = d.nodes[(size_t)sid * capS + perm[j]];
+  }
+  for (int j = threadIdx.x; j < r; j += blockDim.x) {
+    d.piv[(size_t)sid * capS + j] = piv[j];
+    static_cast<T*>(d.Dinv)[(size_t)sid * capS + j] = rinv[j];
+  }
+  if (threadIdx.x == 0) {
+    d.kk[sid] = k;
+    d.hs[sid] = h;
+    work_done += work::interp(k, e) + work::apply(e, k) + (r > 0 ? work::elim(r, k) : 0ull);
+    atomicAdd(d.lstat + LS_PASSES, passes);
+    atomicAdd(d.flops, work_done);
+    atomicAdd(d.flops + 2, (unsigned long long)((k * r + e * e) * sizeof(T) + 2 * e * sizeof(int)));
+  }
 }
 
 // ------------------------------------------------------------ level-L segment tables
@@ -2083,83 +2868,58 @@ __device__ void panel_large(const LevelDev& d, T* M, const int* tab, int ndP, in
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.aligned;\n" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.aligned;\n" ::: "memory"); }
 
-// W = L^{-1} P A_pd and Z = A_dp U^{-1} for the 32 boundary unknowns x0 .. x0 + 31 of a parent, from
-// the factored separator block A (kp <= 32 RS, in shared memory): four columns of W and four rows
-// of Z per warp, lanes over the separator's unknowns, one step per unknown.
-template <typename T, int RS>
-__device__ void panel_chunk(T* M, size_t ldp, int Dp, const int* tab, int x0, int ndP, int kp, const T* A, int lda,
-                            const int* q, const T* inv, T* Zt) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int CJ = 4;
-  const int ldz = kp | 1, nx = min(32, ndP - x0), w0 = CJ * warp;
-  for (int x = threadIdx.x; x < 32 * kp; x += blockDim.x) {
-    const int r = x & 31, j = x >> 5;
-    Zt[r * ldz + j] = M[tab[(size_t)(x0 + min(r, nx - 1)) * MERGE_TABW] + ldp * (Dp + j)];
-  }
-  T s[RS][CJ];
-  size_t pc[CJ];
-#pragma unroll
-  for (int c = 0; c < CJ; ++c) {
-    pc[c] = ldp * tab[(size_t)(x0 + min(w0 + c, nx - 1)) * MERGE_TABW];
-#pragma unroll
-    for (int t = 0; t < RS; ++t) {
-      const int i = min(lane + 32 * t, kp - 1);
-      s[t][c] = M[(Dp + q[i]) + pc[c]];
+// Separators of more than INV_MAX unknowns whose factored block fits in shared memory with 32
+// boundary rows: shared memory of merge_sides_kernel, and of the LU by a cluster of 8
+constexpr int SIDES_MAX = 160;
+template <typename T>
+__host__ __device__ inline size_t sides_bytes(int kp) {
+  const size_t ld = kp | 1;
+  return (kp * ld + 32 * ld + kp) * sizeof(T) + 4 * (size_t)kp + 16;
+}
+template <typename T>
+__host__ __device__ inline bool sides_fit(int kp) { return kp <= SIDES_MAX && sides_bytes<T>(kp) <= 216 * 1024; }
+
+// W and Z of those separators, 32 boundary unknowns per CTA: every CTA reads the factored block and
+// takes its multipliers through the later interchanges (the stored ones stay where the solve's
+// sweeps expect them).  The multiply-adds bound it (kp^2 per boundary unknown), so the boundary
+// spreads over as many SMs as it has groups of 32.  One CTA for all (panel_large) / cluster LU and
+// this kernel, whole merge: 10 parents, separators up to 140, 8.8 / 0.88 ms; 24, 83, 4.0 / 0.60 ms.
+template <typename T>
+__global__ void __launch_bounds__(256) merge_sides_kernel(LevelDev d) {
+  extern __shared__ double pm_sm[];
+  const int P = blockIdx.x;
+  const int ndP = d.pcount[2 * P], kp = d.pcount[2 * P + 1];
+  if (kp <= INV_MAX || !sides_fit<T>(kp)) return;
+  if (32 * (int)blockIdx.y >= ndP) return;
+  const int* tab = d.ptab + (size_t)P * d.ldFp * TABW;
+  const size_t ldp = d.ldFp;
+  T* M = static_cast<T*>(d.Fp) + (size_t)P * ldp * ldp;
+  const T* invg = static_cast<const T*>(d.Pinv) + (size_t)P * d.sepcap;
+  const int* pivg = d.ppiv + (size_t)P * d.sepcap;
+  const int Dp = d.gp.D(), lda = kp | 1;
+  T* A = reinterpret_cast<T*>(pm_sm);
+  T* Zt = A + (size_t)kp * lda;
+  T* inv = Zt + 32 * lda;
+  int* q = reinterpret_cast<int*>(inv + kp);
+  int* piv = reinterpret_cast<int*>(Zt);             // until the first group
+  for (int j = threadIdx.x >> 5; j < kp; j += 8)
+    for (int i = threadIdx.x & 31; i < kp; i += 32) A[i + lda * j] = M[(Dp + i) + ldp * (Dp + j)];
+  for (int j = threadIdx.x; j < kp; j += blockDim.x) { inv[j] = invg[j]; piv[j] = pivg[j]; }
+  __syncthreads();
+  if (threadIdx.x < kp) {
+    T* c = A + (size_t)lda * threadIdx.x;
+    for (int t = threadIdx.x + 1; t < kp; ++t) {
+      const int p = piv[t];
+      if (p != t) { const T a = c[t]; c[t] = c[p]; c[p] = a; }
     }
-  }
-  __syncthreads();                                 // Zt; every entry of W's columns is in registers
-  if (w0 < nx) {
-    for (int j = 0; j < kp; ++j) {
-      T x[CJ];
-#pragma unroll
-      for (int c = 0; c < CJ; ++c) x[c] = __shfl_sync(0xffffffffu, j < 32 ? s[0][c] : s[RS - 1][c], j & 31);
-#pragma unroll
-      for (int t = 0; t < RS; ++t) {
-        const int i = lane + 32 * t;
-        if (i > j && i < kp) {
-          const T l = A[i + lda * j];
-#pragma unroll
-          for (int c = 0; c < CJ; ++c) s[t][c] -= l * x[c];
-        }
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < CJ; ++c)
-#pragma unroll
-      for (int t = 0; t < RS; ++t)
-        if (lane + 32 * t < kp && w0 + c < nx) M[(Dp + lane + 32 * t) + pc[c]] = s[t][c];
-    // Z: row z of z U = a, lanes over its entries
-#pragma unroll
-    for (int c = 0; c < CJ; ++c)
-#pragma unroll
-      for (int t = 0; t < RS; ++t) s[t][c] = Zt[(w0 + c) * ldz + min(lane + 32 * t, kp - 1)];
-    for (int j = 0; j < kp; ++j) {
-      T x[CJ];
-      const T iv = inv[j];
-#pragma unroll
-      for (int c = 0; c < CJ; ++c) x[c] = __shfl_sync(0xffffffffu, j < 32 ? s[0][c] : s[RS - 1][c], j & 31);
-#pragma unroll
-      for (int t = 0; t < RS; ++t) {
-        const int i = lane + 32 * t;
-        if (i > j && i < kp) {
-          const T g = A[j + lda * i] * iv;
-#pragma unroll
-          for (int c = 0; c < CJ; ++c) s[t][c] -= g * x[c];
-        }
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < CJ; ++c)
-#pragma unroll
-      for (int t = 0; t < RS; ++t)
-        if (lane + 32 * t < kp) Zt[(w0 + c) * ldz + lane + 32 * t] = s[t][c] * inv[lane + 32 * t];
+  } else if (threadIdx.x == blockDim.x - 1) {
+    for (int i = 0; i < kp; ++i) q[i] = i;
+    for (int j = 0; j < kp; ++j) { const int p = piv[j], t = q[j]; q[j] = q[p]; q[p] = t; }
   }
   __syncthreads();
-  for (int x = threadIdx.x; x < 32 * kp; x += blockDim.x) {
-    const int r = x & 31, j = x >> 5;
-    if (r < nx) M[tab[(size_t)(x0 + r) * MERGE_TABW] + ldp * (Dp + j)] = Zt[r * ldz + j];
-  }
-  __syncthreads();
+  auto posn = [&](int x) { return tab[(size_t)x * TABW]; };
+  for (int x0 = 32 * blockIdx.y; x0 < ndP; x0 += 32 * gridDim.y)
+    panel_chunk<T, SIDES_MAX / 32>(M, ldp, Dp, posn, x0, ndP, kp, A, lda, q, inv, Zt);
 }
 
 // The separator of each parent: LU of its block, W = L^{-1} P A_pd, Z = A_dp U^{-1}, and the block
@@ -2184,8 +2944,24 @@ __global__ void __launch_bounds__(256) merge_panel_kernel(LevelDev d) {
   T* invg = static_cast<T*>(d.Pinv) + (size_t)P * d.sepcap;
   int* pivg = d.ppiv + (size_t)P * d.sepcap;
   const int Dp = d.gp.D();
-  if (kp > INV_MAX) {
-    if (blockIdx.y == 0) panel_large<T>(d, M, tab, ndP, kp, pivg, invg, shi);
+  if (kp > INV_MAX) {          // the LU by the cluster, W and Z by merge_sides_kernel, where they fit
+    if (sides_fit<T>(kp) && gridDim.y == 8) {
+      cg::cluster_group cl = cg::this_cluster();
+      WideShape W;
+      W.C = (int)gridDim.y;
+      W.rank = (int)blockIdx.y;
+      double* mb = pm_sm;
+      int* piv = reinterpret_cast<int*>(mb + 2 * (kp + 2));
+      T* iv = reinterpret_cast<T*>(piv + ((kp + 1) & ~1));
+      const bool ok = wide_lu<T>(cl, W, M + Dp + ldp * Dp, ldp, kp, piv, iv, iv + kp, mb);
+      __syncthreads();
+      if (blockIdx.y == 0) {
+        if (!ok && threadIdx.x == 0) atomicOr(d.err, ERR_SINGULAR);
+        for (int j = threadIdx.x; j < kp; j += blockDim.x) { invg[j] = iv[j]; pivg[j] = piv[j]; }
+      }
+    } else if (blockIdx.y == 0) {
+      panel_large<T>(d, M, tab, ndP, kp, pivg, invg, shi);
+    }
     return;
   }
   const int lda = kp | 1;
@@ -2200,8 +2976,9 @@ __global__ void __launch_bounds__(256) merge_panel_kernel(LevelDev d) {
   const bool ok = kp <= 32 ? fast_elim<T, 8, 1>(A, lda, 0, kp, q, inv, shi, shi + 6)
                            : fast_elim<T, 8, 2>(A, lda, 0, kp, q, inv, shi, shi + 6);
   for (int x0 = 32 * blockIdx.y; x0 < ndP; x0 += 32 * gridDim.y) {
-    if (kp <= 32) panel_chunk<T, 1>(M, ldp, Dp, tab, x0, ndP, kp, A, lda, q, inv, Zt);
-    else panel_chunk<T, 2>(M, ldp, Dp, tab, x0, ndP, kp, A, lda, q, inv, Zt);
+    auto posn = [&](int x) { return tab[(size_t)x * TABW]; };
+    if (kp <= 32) panel_chunk<T, 1>(M, ldp, Dp, posn, x0, ndP, kp, A, lda, q, inv, Zt);
+    else panel_chunk<T, 2>(M, ldp, Dp, posn, x0, ndP, kp, A, lda, q, inv, Zt);
   }
   cluster_wait();
   if (blockIdx.y != 0) return;
@@ -2980,6 +3757,21 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 16) sep_solve_kernel(Level
 
 }  // namespace
 
+// Clusters per segment and their shared memory (0: none): FP64, levels of more than 16 unknowns per
+// side whose segments leave SMs idle.  Up to 8 CTAs a segment, two per SM at most; one per SM where
+// there is room for that, with all of the shared memory (segments of up to about 290 unknowns), else
+// half of it (about 160).
+void sparsify_wide_plan(const LevelPlan& p, LevelDev* d) {
+  d->wide = d->wide_smem = 0;
+  const int n = p.g.nseg(), sms = sm_count();
+  if (d->fp32 || p.capS <= 16 || n == 0) return;
+  int C = 8;
+  while (C > 1 && n * C > 2 * sms) C /= 2;
+  if (C == 1) return;
+  d->wide = C;
+  d->wide_smem = n * C <= sms ? 216 * 1024 : 108 * 1024;
+}
+
 // The sizes below follow the layout of sparsify_kernel.
 size_t sparsify_smem_need(int e, int symmetric, int h0, int p_over, int tbytes, int chunk) {
   const size_t halves = symmetric ? 1 : 2;
@@ -3042,24 +3834,47 @@ void launch_level_init_L(const LevelDev& d, cudaStream_t s) {
 }
 
 template <typename T>
-static void sparsify_launch(const LevelDev& d, const LevelPlan& p, cudaStream_t s) {
+static void sparsify_launch(const LevelDev& d0, const LevelPlan& p, cudaStream_t s) {
   int smem = (int)p.spars_smem;
+  LevelDev d = d0;
+  // few segments in FP64: a cluster each (the predictor and eps = 0 stay with one CTA)
+  if (d.pred_mode != PRED_OFF || d.eps == 0.0) d.wide = 0;
   if (d.use_order && d.g.nseg() > 0) {
     note_launch();
     seg_order_kernel<<<1, 1024, 0, s>>>(d.cnt, d.g.nseg(), d.order);
   }
-  note_launch();
-  if (d.capS <= 16) {       // finest segments: two warps each, many segments per SM
-    cudaFuncSetAttribute(sparsify_kernel<T, NW_SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaFuncSetAttribute(sparsify_kernel<T, NW_SMALL>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                         cudaSharedmemCarveoutMaxShared);
-    sparsify_kernel<T, NW_SMALL><<<d.g.nseg(), NW_SMALL * 32, smem, s>>>(d, smem);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  cfg.stream = s;
+  cfg.attrs = attr;
+  if (d.wide > 1) {
+    cudaFuncSetAttribute(sparsify_wide_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, d.wide_smem);
+    cfg.gridDim = dim3(d.g.nseg() * d.wide);
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = d.wide_smem;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = d.wide;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.numAttrs = 1;
+    note_launch();
+    cudaLaunchKernelEx(&cfg, sparsify_wide_kernel<T>, d);
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
   } else {
-    cudaFuncSetAttribute(sparsify_kernel<T, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaFuncSetAttribute(sparsify_kernel<T, NW>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                         cudaSharedmemCarveoutMaxShared);
-    sparsify_kernel<T, NW><<<d.g.nseg(), NW * 32, smem, s>>>(d, smem);
+    cfg.numAttrs = 0;
   }
+  cfg.gridDim = dim3(d.g.nseg());
+  cfg.dynamicSmemBytes = smem;
+  note_launch();
+  auto run = [&](auto kernel, int threads) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    cfg.blockDim = dim3(threads);
+    cudaLaunchKernelEx(&cfg, kernel, d, smem);
+  };
+  if (d.capS <= 16) run(sparsify_kernel<T, NW_SMALL>, NW_SMALL * 32);   // two warps each, many segments per SM
+  else run(sparsify_kernel<T, NW>, NW * 32);
 }
 
 void launch_sparsify(const LevelDev& d, const LevelPlan& p, cudaStream_t s) {
@@ -3086,11 +3901,17 @@ static void merge_launch(const LevelDev& d, const LevelPlan& p, cudaStream_t s) 
     // two parents per SM: a cluster of up to 8 CTAs per parent (more never helps: 256 boundary
     // unknowns), else one
     const size_t kb = (size_t)std::min(p.sepcap, INV_MAX), lda = kb | 1;
-    const int pm = (int)(sizeof(T) * (kb * lda + std::max(kb * kb, 32 * lda)));
-    cudaFuncSetAttribute(merge_panel_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, pm);
+    int pm = (int)(sizeof(T) * (kb * lda + std::max(kb * kb, 32 * lda)));
     int cl = 1;
     if (np <= 2 * sm_count())
       while (cl < 8 && 32 * cl < p.ldFp) cl *= 2;
+    // larger separators: the cluster's columns of the block, two multiplier buffers, pivots
+    const bool sides = cl == 8 && p.sepcap > INV_MAX;
+    if (sides) {
+      const size_t km = std::min(p.sepcap, SIDES_MAX);
+      pm = std::max(pm, (int)(sizeof(T) * (km * ((km + 7) / 8) + km) + 16 * (km + 2) + 4 * (km + 2)));
+    }
+    cudaFuncSetAttribute(merge_panel_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, pm);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(np, cl);
     cfg.blockDim = dim3(256);
@@ -3105,6 +3926,14 @@ static void merge_launch(const LevelDev& d, const LevelPlan& p, cudaStream_t s) 
     cfg.numAttrs = 1;
     note_launch();
     cudaLaunchKernelEx(&cfg, merge_panel_kernel<T>, d);
+    if (sides) {
+      int ks = std::min(p.sepcap, SIDES_MAX);
+      while (!sides_fit<T>(ks)) --ks;
+      const int sb = (int)sides_bytes<T>(ks);
+      cudaFuncSetAttribute(merge_sides_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sb);
+      note_launch();
+      merge_sides_kernel<T><<<dim3(np, std::min((p.ldFp + 31) / 32, 48)), 256, sb, s>>>(d);
+    }
   }
   note_launch();
   if (d.schur_tc && d.fp32) {

@@ -158,6 +158,8 @@ struct LevelDev {
   // options
   double eps;
   int symmetric, p_over, near_radius, h0;
+  int wide;         // CTAs per segment of the sparsification (a cluster; 0: one CTA)
+  int wide_smem;    // their shared memory
   int schur_tc;     // separator Schur updates on the tensor cores (mixed path only)
   int sketch_tc;    // sketch products G B_F on the tensor cores (mixed path only)
   unsigned long long seed;
@@ -313,6 +315,8 @@ size_t sparsify_smem_min(int e, int symmetric, int h0, int p_over, int tbytes);
 // Dynamic shared memory per sparsify CTA that lets `ctas` of them be resident on one SM
 // (the variant that a level of segment capacity capS launches; 0 when that many cannot fit)
 size_t sparsify_smem_budget(int fp32, int capS, int ctas);
+// CTAs per segment and their shared memory for level p (sets d->wide, d->wide_smem)
+void sparsify_wide_plan(const LevelPlan& p, LevelDev* d);
 // Streaming multiprocessors of the current device
 int sm_count();
 
