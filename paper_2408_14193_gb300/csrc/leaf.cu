@@ -339,9 +339,47 @@ __device__ __forceinline__ void sweep_U(const BandT& B, In in, Out out) {
 // slot c mod WS; after step j column j is final, goes to global memory in precision T and its
 // slot is refilled with column j + WS (first touched at step j + 2) from the gathered nonzeros
 // (leaf_band5_kernel) by cp.async, waited for two steps later.
-// Also zeroes the leaf's frontal block and records the upper bandwidth reached.
+// Also zeroes the leaf's frontal block, where `couple` is set puts the couplings that it owns there
+// (the Schur kernel over the band rows subtracts from them), and records the upper bandwidth reached.
 constexpr int WS = 32;       // window columns (> KV)
 constexpr int LUT = 64;      // threads per leaf LU
+
+template <typename T>
+__device__ __forceinline__ void own_couplings(const LeafDev& d, int b, int tid, T* F) {
+  const int nx = d.nx, x0 = (b % d.g.bx) * (LEAF + 1), y0 = (b / d.g.bx) * (LEAF + 1);
+  // original couplings owned by this box: its TOP and RIGHT sides (it is their lower /
+  // left box) with their end junctions, and the diagonal of its BL junction.
+  //   task 0..14 TOP row -> TOP, TL, TR   15..29 RIGHT row -> RIGHT, BR, TR
+  //   30 TL row -> TOP   31 TR row -> TOP, RIGHT   32 BR row -> RIGHT   33 BL row -> BL
+  if (tid < 2 * LEAF + 4) {
+    int vx, vy;
+    if (tid < LEAF) { vx = x0 + tid; vy = y0 + LEAF; }
+    else if (tid < 2 * LEAF) { vx = x0 + LEAF; vy = y0 + tid - LEAF; }
+    else if (tid == 30) { vx = x0 - 1; vy = y0 + LEAF; }
+    else if (tid == 31) { vx = x0 + LEAF; vy = y0 + LEAF; }
+    else if (tid == 32) { vx = x0 + LEAF; vy = y0 - 1; }
+    else { vx = x0 - 1; vy = y0 - 1; }
+    if (vx >= 0 && vx < nx && vy >= 0 && vy < d.ny) {
+      const int row = vx + nx * vy;
+      const int pi = leaf_frontal_pos(vx, vy, x0, y0);
+      for (int p = d.rowptr[row]; p < d.rowptr[row + 1]; ++p) {
+        int c = d.colind[p];
+        int pj = leaf_frontal_pos(c % nx, c / nx, x0, y0);
+        if (pj < 0) continue;
+        const bool on_top = pj >= LEAF && pj < 2 * LEAF;
+        const bool on_right = pj >= 3 * LEAF && pj < 4 * LEAF;
+        bool take;
+        if (tid < LEAF) take = on_top || pj == 4 * LEAF + C_TL || pj == 4 * LEAF + C_TR;
+        else if (tid < 2 * LEAF) take = on_right || pj == 4 * LEAF + C_BR || pj == 4 * LEAF + C_TR;
+        else if (tid == 30) take = on_top;
+        else if (tid == 31) take = on_top || on_right;
+        else if (tid == 32) take = on_right;
+        else take = (pj == pi);
+        if (take) F[pi + (size_t)d.ldF * pj] += (T)d.val[p];
+      }
+    }
+  }
+}
 
 // The leaf matrices' nonzeros by column, gathered from the CSR once for all leaves (one thread
 // per leaf, column and stencil offset, every lookup independent), so that the LU's window
@@ -365,7 +403,7 @@ __global__ void leaf_band5_kernel(LeafDev d) {
 }
 
 template <typename T>
-__global__ void __launch_bounds__(LUT) leaf_lu_kernel(LeafDev d) {
+__global__ void __launch_bounds__(LUT) leaf_lu_kernel(LeafDev d, int couple) {
   __shared__ double W[LDAB * WS];
   __shared__ int sh[2];
   const int b = blockIdx.x;
@@ -453,6 +491,7 @@ __global__ void __launch_bounds__(LUT) leaf_lu_kernel(LeafDev d) {
     cp_async_commit();
   }
   cp_async_wait<0>();
+  if (couple) own_couplings<T>(d, b, tid, reinterpret_cast<T*>(d.F) + (size_t)b * d.ldF * d.ldF);
   if (!ok && tid == 0) atomicOr(d.err, ERR_SINGULAR);
   if (tid == 0) {
     const int ku = min(kureach, KV);
@@ -554,38 +593,7 @@ __global__ void __launch_bounds__(FTH) leaf_schur_kernel(LeafDev d) {
   }
   __syncthreads();
   const bool active = live;
-  // original couplings owned by this box: its TOP and RIGHT sides (it is their lower /
-  // left box) with their end junctions, and the diagonal of its BL junction.
-  //   task 0..14 TOP row -> TOP, TL, TR   15..29 RIGHT row -> RIGHT, BR, TR
-  //   30 TL row -> TOP   31 TR row -> TOP, RIGHT   32 BR row -> RIGHT   33 BL row -> BL
-  if (active && tid < 2 * LEAF + 4) {
-    int vx, vy;
-    if (tid < LEAF) { vx = x0 + tid; vy = y0 + LEAF; }
-    else if (tid < 2 * LEAF) { vx = x0 + LEAF; vy = y0 + tid - LEAF; }
-    else if (tid == 30) { vx = x0 - 1; vy = y0 + LEAF; }
-    else if (tid == 31) { vx = x0 + LEAF; vy = y0 + LEAF; }
-    else if (tid == 32) { vx = x0 + LEAF; vy = y0 - 1; }
-    else { vx = x0 - 1; vy = y0 - 1; }
-    if (vx >= 0 && vx < nx && vy >= 0 && vy < d.ny) {
-      const int row = vx + nx * vy;
-      const int pi = leaf_frontal_pos(vx, vy, x0, y0);
-      for (int p = d.rowptr[row]; p < d.rowptr[row + 1]; ++p) {
-        int c = d.colind[p];
-        int pj = leaf_frontal_pos(c % nx, c / nx, x0, y0);
-        if (pj < 0) continue;
-        const bool on_top = pj >= LEAF && pj < 2 * LEAF;
-        const bool on_right = pj >= 3 * LEAF && pj < 4 * LEAF;
-        bool take;
-        if (tid < LEAF) take = on_top || pj == 4 * LEAF + C_TL || pj == 4 * LEAF + C_TR;
-        else if (tid < 2 * LEAF) take = on_right || pj == 4 * LEAF + C_BR || pj == 4 * LEAF + C_TR;
-        else if (tid == 30) take = on_top;
-        else if (tid == 31) take = on_top || on_right;
-        else if (tid == 32) take = on_right;
-        else take = (pj == pi);
-        if (take) F[pi + (size_t)d.ldF * pj] += (T)d.val[p];
-      }
-    }
-  }
+  if (active) own_couplings<T>(d, b, tid, F);
 }
 
 // ---------------------------------------------------------------- solve
@@ -961,15 +969,16 @@ __device__ __forceinline__ void rows_load_U(const double* ur, int blk, int l, do
   for (int u = 0; u < 16; ++u) v[u] = __ldg(ur + 16 * min(16 * bk + u, NI - 1) + ((u - l + 16) & 15));
 }
 
-// y = L^{-1} P y in place (y: R columns of RROW values, rows >= NI zero).  lv holds block 0.
+// y = L^{-1} P y in place (y: R columns of RROW values, rows >= NI zero; rows before block b0 stay
+// as they are).  lv holds block b0.
 template <int R, bool PIV>
-__device__ __forceinline__ void rows_sweep_L(const double* lr, double* y, double (&lv)[16]) {
+__device__ __forceinline__ void rows_sweep_L(const double* lr, double* y, double (&lv)[16], int b0) {
   const int lane = threadIdx.x & 31, l = lane & 15, hb = lane & 16;
   double W[R];
 #pragma unroll
-  for (int c = 0; c < R; ++c) W[c] = y[c * RROW + l];
+  for (int c = 0; c < R; ++c) W[c] = y[c * RROW + 16 * b0 + l];
 #pragma unroll 1
-  for (int blk = 0; blk < RNB; ++blk) {
+  for (int blk = b0; blk < RNB; ++blk) {
     double ln[16], nx[R], fin[R];
     rows_load_L(lr, blk + 1, l, ln);
 #pragma unroll
@@ -1123,7 +1132,7 @@ __global__ void __launch_bounds__(RWPB * 32) leaf_rows_kernel(LeafDev d, double*
 #pragma unroll
     for (int c = 0; c < R; ++c) y[c * RROW + jr] = v[c];
   }
-  rows_sweep_L<R, WIDE>(lr, y, lv);
+  rows_sweep_L<R, WIDE>(lr, y, lv, 0);
   rows_sweep_U<R, WIDE>(ur, ux, y);
   if (!live) return;
 #pragma unroll 1
@@ -1136,6 +1145,76 @@ __global__ void __launch_bounds__(RWPB * 32) leaf_rows_kernel(LeafDev d, double*
         if constexpr (!bwd) *x = y[c * RROW + j];
         else *x -= y[c * RROW + j];
       }
+  }
+}
+
+// ---- leaf factorization, kernel B in FP64: the sweeps over the band rows, R of the 60 columns per
+// half-warp.  The columns are taken in the order of their interior neighbours' rows m and a warp
+// starts its L sweep at the block of 16 rows that holds the first of them (15 rows earlier where
+// the leaf has interchanges: they move a row up by at most 15).  The leaf's couplings are in F
+// already; a column of F takes A_dI times the ring of its solution.
+// For grids of few leaves: there the chain of a thread that owns a column bounds the time (31 FP64
+// instructions of 64 cycles for a step of L and one of U), here it is 2 R + 1.  At 32 leaves the
+// leaf factorization takes 325 us with it and 575 without.  On many leaves both forms
+// are bound by the FP64 pipe and this one issues more (the scaled U column, the halves' idle lanes).
+template <int R>
+__host__ __device__ constexpr int schur_warps() { return R == 2 ? 3 : 2; }          // per CTA
+template <int R>
+__host__ __device__ constexpr int schur_ctas() { return NQ / (2 * R * schur_warps<R>()); }   // per leaf
+template <int R>
+__global__ void __launch_bounds__(schur_warps<R>() * 32) leaf_schur_rows_kernel(LeafDev d) {
+  static_assert(schur_ctas<R>() * schur_warps<R>() * 2 * R == NQ, "columns dealt out evenly");
+  extern __shared__ float4 lsm4[];
+  __shared__ double qa[NQ], qc[NQ];
+  __shared__ int qm[NQ], qex[NQ];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane >> 4, l = lane & 15;
+  const int b = blockIdx.x / schur_ctas<R>(), part = blockIdx.x % schur_ctas<R>();
+  const int nx = d.nx, x0 = (b % d.g.bx) * (LEAF + 1), y0 = (b / d.g.bx) * (LEAF + 1);
+  const double* lr = reinterpret_cast<const double*>(d.lrec) + (size_t)b * NI * 16;
+  const double* ur = reinterpret_cast<const double*>(d.urec) + (size_t)b * NI * 16;
+  const double* ux = reinterpret_cast<const double*>(d.uext) + (size_t)b * NI * 16;
+  for (int q = threadIdx.x; q < NQ; q += blockDim.x) {
+    int vx, vy, m;
+    side_unknown(q, x0, y0, &vx, &vy, &m);
+    const bool exists = vx >= 0 && vx < nx && vy >= 0 && vy < d.ny;
+    double a = 0.0, c = 0.0;
+    if (exists) {
+      const int node = vx + nx * vy, mnode = (x0 + m % LEAF) + nx * (y0 + m / LEAF);
+      a = csr_entry(d.rowptr, d.colind, d.val, node, mnode);
+      c = csr_entry(d.rowptr, d.colind, d.val, mnode, node);
+    }
+    qm[q] = m;
+    qex[q] = exists ? 1 : 0;
+    qa[q] = a;
+    qc[q] = c;
+    if (part == 0) reinterpret_cast<double*>(d.cpl)[(size_t)b * NQ + q] = c;   // 0 outside the grid
+  }
+  double* y = reinterpret_cast<double*>(lsm4) + (2 * warp + sub) * row_leaf_pitch<R>();
+  for (int x = l; x < R * RROW; x += 16) y[x] = 0.0;
+  __syncthreads();
+  const int first = (part * schur_warps<R>() + warp) * 2 * R;    // place of the warp's first column
+  const int q0 = first + sub * R;                                // ... of the half-warp's
+  if (l < R) {
+    const int q = c_qorder[q0 + l];
+    y[l * RROW + qm[q]] = qc[q];
+  }
+  __syncwarp();
+  const bool piv = *d.kumax > 15;                                // some leaf made an interchange
+  const int m0 = qm[c_qorder[first]], b0 = (piv ? max(m0 - 15, 0) : m0) / 16;
+  double lv[16];
+  rows_load_L(lr, b0, l, lv);
+  if (piv) rows_sweep_L<R, true>(lr, y, lv, b0);
+  else rows_sweep_L<R, false>(lr, y, lv, b0);
+  if (d.kur[b] > 15) rows_sweep_U<R, true>(ur, ux, y);
+  else rows_sweep_U<R, false>(ur, ux, y);
+  __syncwarp();
+  double* F = reinterpret_cast<double*>(d.F) + (size_t)b * d.ldF * d.ldF;
+#pragma unroll 1
+  for (int c = 0; c < R; ++c) {
+    const int q = c_qorder[q0 + c];
+    if (!qex[q]) continue;
+    for (int r = l; r < NQ; r += 16)
+      if (qex[r]) F[r + (size_t)d.ldF * q] -= qa[r] * y[c * RROW + qm[r]];
   }
 }
 
@@ -1322,6 +1401,22 @@ cudaError_t leaf_init_tables() {
   return e;
 }
 
+template <int R>
+static void leaf_schur_rows_go(const LeafDev& d, cudaStream_t s) {
+  const int smem = (int)(2 * schur_warps<R>() * row_leaf_pitch<R>() * sizeof(double));
+  cudaFuncSetAttribute(leaf_schur_rows_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  leaf_schur_rows_kernel<R><<<d.g.nbox() * schur_ctas<R>(), schur_warps<R>() * 32, smem, s>>>(d);
+}
+
+// Columns per half-warp of the FP64 Schur kernel over the band rows, or 0 for the one with a thread per
+// column.  Leaf factorization, 2 / 5 / thread per column: 16 leaves 321 / 400 / 575 us, 64 375 / 407 /
+// 577, 128 433 / 417 / 578, 256 571 / 572 / 585 (with interchanges 802 / 792 / 872), 1024 1489 / 1210 /
+// 1175, 4096 5559 / 4313 / 3838.
+static int schur_rows_width(int nbox) {
+  const int sms = sm_count();
+  return 2 * nbox <= sms ? 2 : nbox <= 2 * sms ? 5 : 0;
+}
+
 void launch_leaf_factor(const LeafDev& d, cudaStream_t s) {
   const int nbox = d.g.nbox();
   note_launch();
@@ -1332,10 +1427,13 @@ void launch_leaf_factor(const LeafDev& d, cudaStream_t s) {
     leaf_band5_kernel<<<(int)blocks, 256, 0, s>>>(d);
   }
   note_launch();
-  if (d.fp32) leaf_lu_kernel<float><<<nbox, LUT, 0, s>>>(d);
-  else leaf_lu_kernel<double><<<nbox, LUT, 0, s>>>(d);
+  const int R = d.fp32 ? 0 : schur_rows_width(nbox);
+  if (d.fp32) leaf_lu_kernel<float><<<nbox, LUT, 0, s>>>(d, 0);
+  else leaf_lu_kernel<double><<<nbox, LUT, 0, s>>>(d, R > 0);
   note_launch();
   if (d.fp32) leaf_schur_kernel<float><<<(nbox + LPC - 1) / LPC, FTH, 0, s>>>(d);
+  else if (R == 2) leaf_schur_rows_go<2>(d, s);
+  else if (R == 5) leaf_schur_rows_go<5>(d, s);
   else leaf_schur_kernel<double><<<(nbox + LPC - 1) / LPC, FTH, 0, s>>>(d);
 }
 
