@@ -88,10 +88,6 @@ struct Band {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
-__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem));
-}
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem));
@@ -334,15 +330,20 @@ __device__ __forceinline__ void sweep_U(const BandT& B, In in, Out out) {
 
 // ---- leaf factorization, kernel A: band LU (the dgbtf2 sequence: pivot = largest |entry| of
 // the column inside the band, ties -> lowest row; interchanges applied to the columns the U
-// factor can reach; multipliers scaled by the reciprocal pivot) of one leaf per 64-thread
-// CTA, in FP64, on a sliding window of WS band columns in shared memory: column c sits in
-// slot c mod WS; after step j column j is final, goes to global memory in precision T and its
-// slot is refilled with column j + WS (first touched at step j + 2) from the gathered nonzeros
-// (leaf_band5_kernel) by cp.async, waited for two steps later.
+// factor can reach; multipliers scaled by the reciprocal pivot) of one leaf per CTA, in FP64,
+// on a sliding window of WS band columns in shared memory: column c sits in slot c mod WS.
+// One barrier per pivot: at step j a half-warp holds a column (lanes over the 15 rows below j) and
+// applies interchange and rank-1 update to it; warp 0 takes column j + 1, which it keeps in
+// registers, finds its pivot, scales it and leaves it ready for the next step, while the other
+// warps finish the columns from j + 3 on.  The last warp also stores column j - 1, final since
+// the barrier, and refills its slot with column j + 31 (first touched at step j + 1) from the
+// gathered nonzeros (leaf_band5_kernel), loaded a step ahead.
+// What bounds it: with few leaves the chain from pivot to pivot (an update, three warp
+// reductions, a FP64 reciprocal of about 370 cycles, the scaling); with many the FP64 pipe (18
+// instructions of 64 cycles a step, half of them the reciprocal's).
 // Also zeroes the leaf's frontal block, where `couple` is set puts the couplings that it owns there
 // (the Schur kernel over the band rows subtracts from them), and records the upper bandwidth reached.
 constexpr int WS = 32;       // window columns (> KV)
-constexpr int LUT = 64;      // threads per leaf LU
 
 template <typename T>
 __device__ __forceinline__ void own_couplings(const LeafDev& d, int b, int tid, T* F) {
@@ -402,12 +403,14 @@ __global__ void leaf_band5_kernel(LeafDev d) {
   }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(LUT) leaf_lu_kernel(LeafDev d, int couple) {
+template <typename T, int LUW>
+__global__ void __launch_bounds__(32 * LUW) leaf_lu_kernel(LeafDev d, int couple) {
+  constexpr int LUT = 32 * LUW;
   __shared__ double W[LDAB * WS];
-  __shared__ int sh[2];
+  __shared__ double rps[4];    // of the last pivots: reciprocal, offset, whether zero
+  __shared__ int offs[4], zeros[4];
   const int b = blockIdx.x;
-  const int tid = threadIdx.x, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const Geo g = d.g;
   {
     T* F = reinterpret_cast<T*>(d.F) + (size_t)b * d.ldF * d.ldF;
@@ -426,71 +429,97 @@ __global__ void __launch_bounds__(LUT) leaf_lu_kernel(LeafDev d, int couple) {
   };
   auto w = [&](int i, int c) -> double& { return W[(KV + i - c) + LDAB * (c & (WS - 1))]; };
   for (int x = tid; x < LDAB * WS; x += LUT) W[x] = assemble(x % LDAB, x / LDAB);
-  // band row tid of a refilled column: stencil offset k of the gathered nonzeros, or none
-  const int ko = tid - KV;
-  const int kst = ko == -LEAF ? 0 : ko == -1 ? 1 : ko == 0 ? 2 : ko == 1 ? 3 : ko == LEAF ? 4 : -1;
+  // pivot of column c: a is its entry in row c + lane (lanes 0 .. 15 of warp 0)
+  auto pivot = [&](int c, double a) {
+    const int km = min(KL, NI - 1 - c);
+    const bool in = lane <= km;
+    const unsigned ah = (unsigned)((unsigned long long)__double_as_longlong(a) >> 32) & 0x7fffffffu;
+    const unsigned al = (unsigned)(unsigned long long)__double_as_longlong(a);
+    const unsigned hi = __reduce_max_sync(0xffffffffu, in ? ah : 0u);
+    const unsigned lo = __reduce_max_sync(0xffffffffu, in && ah == hi ? al : 0u);
+    const int p = (int)__reduce_min_sync(0xffffffffu, in && ah == hi && al == lo ? (unsigned)lane : 31u) & 15;
+    const bool zero = (hi | lo) == 0u;
+    const double pv = __shfl_sync(0xffffffffu, a, p), a0 = __shfl_sync(0xffffffffu, a, 0);
+    const double rp = zero ? 0.0 : 1.0 / pv;
+    const double v = lane == 0 ? pv : lane == p ? a0 : a;
+    if (in) w(c + min(lane, km), c) = lane == 0 || zero ? v : v * rp;
+    if (lane == 0) { rps[c & 3] = rp; offs[c & 3] = p; zeros[c & 3] = zero ? 1 : 0; }
+  };
+  // the last warp's rows of a stored or refilled column: lane, lane + 32
+  auto stencil = [](int t) {
+    const int o = t - KV;
+    return o == -LEAF ? 0 : o == -1 ? 1 : o == 0 ? 2 : o == 1 ? 3 : o == LEAF ? 4 : -1;
+  };
+  const int k0 = stencil(lane), k1 = stencil(lane + 32);
+  double n0 = 0.0, n1 = 0.0;   // column j + 31's entries at step j
+  auto fetch = [&](int c) {
+    const double* q = b5 + 5 * min(c, NI - 1);
+    n0 = k0 >= 0 ? q[k0] : 0.0;
+    n1 = k1 >= 0 ? q[k1] : 0.0;
+  };
+  auto store = [&](int c, int t) {
+    const T v = (T)W[t + LDAB * (c & (WS - 1))];
+    if (t > KV) lrg[16 * c + (t - KV - 1)] = v;                  // L(c+1+r, c), r = t - KV - 1
+    else if (t == KV) {
+      lrg[16 * c + 15] = (T)offs[c & 3];                         // pivot offset 0..15, exact in T
+      urg[16 * c] = (T)rps[c & 3];
+      uxg[16 * c + 15] = T(0);
+    } else if (t > KV - 16) urg[16 * c + (KV - t)] = v;          // U(c-r, c), r = KV - t <= 15
+    else uxg[16 * c + (KV - 16 - t)] = v;                        // U(c-r, c), r = 16..30
+  };
+  __syncthreads();
+  if (warp == 0) pivot(0, w(min(lane, KL), 0));
+  if (warp == LUW - 1) fetch(WS);
   __syncthreads();
   int ju = 0, kureach = KU;
   bool ok = true, swapped = false;
-  const int ur = 1 + (tid & 15), ucg = tid >> 4;       // rank-1 update: row, column group
+  const int r = lane & 15, half = lane >> 4;
   for (int j = 0; j < NI; ++j) {
-    const int km = min(KL, NI - 1 - j);
-    cp_async_wait<1>();       // the refills issued up to step j - 2 (column j + 30 at the latest)
-    if (tid < 32) {           // pivot: |entries| compared as bit patterns (no FP64 arithmetic)
-      long long best = -1;
-      int bi = 0;
-      if (lane <= km) { best = __double_as_longlong(w(j + lane, j)) & 0x7fffffffffffffffll; bi = lane; }
-      for (int o = 16; o > 0; o >>= 1) {
-        const long long ob = __shfl_down_sync(0xffffffffu, best, o);
-        const int oi = __shfl_down_sync(0xffffffffu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-      }
-      if (lane == 0) {
-        sh[0] = bi;
-        sh[1] = best == 0 ? 1 : 0;
-        lrg[16 * j + 15] = (T)bi;      // pivot offset 0..15, exact in T
-      }
-    }
-    __syncthreads();
-    const int jp = sh[0];
-    const bool zero = sh[1] != 0;
+    const int km = min(KL, NI - 1 - j), jp = offs[j & 3];
+    const bool zero = zeros[j & 3] != 0;
     if (zero) ok = false;
     swapped |= jp != 0;
     ju = max(ju, min(j + KU + jp, NI - 1));
     kureach = max(kureach, ju - j);
-    if (!zero && jp != 0)
-      for (int c = j + tid; c <= ju; c += LUT) {
-        const double a = w(j, c);
-        w(j, c) = w(j + jp, c);
-        w(j + jp, c) = a;
+    // row j + 1 + r (lane 15: only kept, for the pivot of column j + 1)
+    const int i = min(j + 1 + r, NI - 1);
+    const double m = r < km && !zero ? w(min(i, j + KL), j) : 0.0;
+    auto update = [&](int c) {               // column c <= ju; the new entry of row i
+      const double a = w(i, c), u = w(j + jp, c), o = w(j, c);
+      __syncwarp();
+      double v = a;
+      if (r < km && !zero) {
+        v = (r + 1 == jp ? o : a) - m * u;
+        w(i, c) = v;
       }
-    __syncthreads();
-    if (tid < 32) {           // one reciprocal per pivot; multipliers scaled by it
-      const double rp = zero ? 0.0 : 1.0 / w(j, j);
-      if (!zero && tid < km) w(j + 1 + tid, j) *= rp;
-      if (tid == 0) urg[16 * j] = (T)rp;
+      if (r == 15) w(j, c) = u;
+      return v;
+    };
+    if (warp == 0) {
+      if (j + 1 < NI) {
+        const double v = update(min(j + 1 + half, NI - 1));
+        __syncwarp();
+        pivot(j + 1, v);
+      }
+    } else {
+      if (warp == LUW - 1 && j > 0) {
+        store(j - 1, lane);
+        if (lane + 32 < LDAB) store(j - 1, lane + 32);
+        if (j - 1 + WS < NI) {
+          W[lane + LDAB * ((j - 1) & (WS - 1))] = n0;
+          if (lane + 32 < LDAB) W[lane + 32 + LDAB * ((j - 1) & (WS - 1))] = n1;
+          fetch(j + WS);
+        }
+        __syncwarp();
+      }
+      for (int c = j + 3 + 2 * (warp - 1); c <= ju; c += 2 * (LUW - 1)) update(min(c + half, ju));
     }
     __syncthreads();
-    if (!zero && ur <= km) {
-      const double m = w(j + ur, j);
-      for (int c = j + 1 + ucg; c <= ju; c += LUT / 16) w(j + ur, c) -= m * w(j, c);
-    }
-    __syncthreads();
-    if (tid < LDAB) {         // column j is final: store its records, refill its slot with column j + WS
-      double& slot = W[tid + LDAB * (j & (WS - 1))];
-      const T v = (T)slot;
-      if (tid > KV) lrg[16 * j + (tid - KV - 1)] = v;              // L(j+1+r, j), r = tid - KV - 1
-      else if (tid > KV - 16) { if (tid < KV) urg[16 * j + (KV - tid)] = v; }   // U(j-r, j), r = KV - tid <= 15
-      else uxg[16 * j + (KV - 16 - tid)] = v;                      // U(j-r, j), r = 16..30
-      if (tid == KV) uxg[16 * j + 15] = T(0);
-      // column j + WS (first touched at step j + 2): its stencil rows copied asynchronously, the
-      // rest zero, so that no global load is outstanding at the next barriers
-      if (j + WS < NI && kst >= 0) cp_async8(&slot, b5 + 5 * (j + WS) + kst);
-      else slot = 0.0;
-    }
-    cp_async_commit();
   }
-  cp_async_wait<0>();
+  if (warp == LUW - 1) {
+    store(NI - 1, lane);
+    if (lane + 32 < LDAB) store(NI - 1, lane + 32);
+  }
   if (couple) own_couplings<T>(d, b, tid, reinterpret_cast<T*>(d.F) + (size_t)b * d.ldF * d.ldF);
   if (!ok && tid == 0) atomicOr(d.err, ERR_SINGULAR);
   if (tid == 0) {
@@ -1417,6 +1446,17 @@ static int schur_rows_width(int nbox) {
   return 2 * nbox <= sms ? 2 : nbox <= 2 * sms ? 5 : 0;
 }
 
+template <int LUW>
+static void leaf_lu_go(const LeafDev& d, int couple, cudaStream_t s) {
+  if (d.fp32) leaf_lu_kernel<float, LUW><<<d.g.nbox(), 32 * LUW, 0, s>>>(d, couple);
+  else leaf_lu_kernel<double, LUW><<<d.g.nbox(), 32 * LUW, 0, s>>>(d, couple);
+}
+
+// Warps per leaf LU.  Leaf factorization with 2 / 3 / 5: 32 leaves 276 / - / 222 us, 256 521 / - / 470;
+// 1024 1162 / 1128 / 1150, 4096 3846 / 3822 / 3875 (more CTAs per SM, a smaller last wave).  Two
+// warps with five barriers a pivot: 32 leaves 325 us, 256 572, 1024 1175, 4096 3838.
+static int lu_warps(int nbox) { return nbox <= 2 * sm_count() ? 5 : 3; }
+
 void launch_leaf_factor(const LeafDev& d, cudaStream_t s) {
   const int nbox = d.g.nbox();
   note_launch();
@@ -1428,8 +1468,8 @@ void launch_leaf_factor(const LeafDev& d, cudaStream_t s) {
   }
   note_launch();
   const int R = d.fp32 ? 0 : schur_rows_width(nbox);
-  if (d.fp32) leaf_lu_kernel<float><<<nbox, LUT, 0, s>>>(d, 0);
-  else leaf_lu_kernel<double><<<nbox, LUT, 0, s>>>(d, R > 0);
+  if (lu_warps(nbox) == 5) leaf_lu_go<5>(d, R > 0, s);
+  else leaf_lu_go<3>(d, R > 0, s);
   note_launch();
   if (d.fp32) leaf_schur_kernel<float><<<(nbox + LPC - 1) / LPC, FTH, 0, s>>>(d);
   else if (R == 2) leaf_schur_rows_go<2>(d, s);
