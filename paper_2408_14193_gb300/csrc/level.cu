@@ -1939,7 +1939,9 @@ __device__ void panel_chunk(T* M, size_t ldp, int Dp, Pos posn, int x0, int ndP,
 // What bounds it: the pivots' serial chain (a cluster barrier, two block reductions, a FP64 square
 // root and a quotient each) and the FP64 pipe of C SMs.  One CTA / cluster, 1023 x 1023 at eps 1e-8:
 // Helmholtz, 10 segments of up to 155 unknowns, 33.2 / 3.6 ms; 24 of up to 101, 10.2 / 1.7 ms;
-// diffusion, 24 of up to 57, 858 / 535 us.
+// diffusion, 24 of up to 57, 858 / 535 us.  FP64 only: in FP32 a segment is not bound by a pipe, and the
+// clusters' barriers cost more than their SMs give (mixed, levels 6 - 2: 169 / 235, 188 / 230, 183 / 238,
+// 142 / 192, 104 / 159 us).
 // Columns: warp w of NSW = min(8, ceil(e / 32)) column sets x RG row groups holds set w mod NSW (and
 // set w + 8 where e > 256), rows r mod RG = w / NSW; the warps of row group 0 own the columns' state.
 namespace cg = cooperative_groups;
@@ -3853,7 +3855,8 @@ static void sparsify_launch(const LevelDev& d0, const LevelPlan& p, cudaStream_t
   cudaLaunchAttribute attr[1];
   cfg.stream = s;
   cfg.attrs = attr;
-  if (d.wide > 1) {
+  cfg.numAttrs = 0;
+  if constexpr (sizeof(T) == 8) if (d.wide > 1) {
     cudaFuncSetAttribute(sparsify_wide_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, d.wide_smem);
     cfg.gridDim = dim3(d.g.nseg() * d.wide);
     cfg.blockDim = dim3(256);
@@ -3867,8 +3870,6 @@ static void sparsify_launch(const LevelDev& d0, const LevelPlan& p, cudaStream_t
     cudaLaunchKernelEx(&cfg, sparsify_wide_kernel<T>, d);
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-  } else {
-    cfg.numAttrs = 0;
   }
   cfg.gridDim = dim3(d.g.nseg());
   cfg.dynamicSmemBytes = smem;
