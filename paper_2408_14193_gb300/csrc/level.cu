@@ -285,7 +285,7 @@ __device__ int block_cpqr(T* Y, int ldy, int m, int e, double eps, int* perm, do
       for (int j = i + lane; j < e; j += 32)
         if (dbits(vn1[j]) >= thr && j < best) best = j;
       for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(0xffffffffu, best, o));
-      if (lane == 0) shi[0] = best;
+      if (lane == 0) shi[0] = best < e ? best : i;     // i: only where a norm is not a number
     }
     __syncthreads();
     const int p = shi[0];
@@ -424,6 +424,7 @@ __device__ bool block_gepp(T* A, int lda, int r0, int n, int ncol, int* piv, T* 
         int oi = __shfl_xor_sync(0xffffffffu, bi, o);
         if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
       }
+      if (bi >= n) bi = j;     // only where no entry of the column is a number
       if (lane == 0) { shi[0] = bi; shi[1] = best == 0.0; piv[j] = bi; }
     }
     __syncthreads();
@@ -2826,6 +2827,7 @@ __device__ void panel_large(const LevelDev& d, T* M, const int* tab, int ndP, in
         int oi = __shfl_xor_sync(0xffffffffu, bi, o);
         if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
       }
+      if (bi >= kp) bi = j;    // only where no entry of the column is a number
       if (lane == 0) { shi[0] = bi; shi[1] = best == 0.0; piv[j] = bi; }
     }
     __syncthreads();
