@@ -235,6 +235,14 @@ __device__ __forceinline__ T bval_q(const LevelDev& d, const SegCtx& S, const T*
 
 // non-negative doubles order like their bit patterns
 __device__ __forceinline__ long long dbits(double x) { return __double_as_longlong(x); }
+// ... a squared norm that is not a number (of either sign) above them all: its column becomes the
+// pivot, and what is not a number reaches R, T and the solution instead of passing for a zero column
+__device__ __forceinline__ long long norm_bits(double x) { return dbits(x) & 0x7fffffffffffffffll; }
+// the smallest pattern that ties with the largest squared norm mx (a pattern)
+__device__ __forceinline__ long long tie_bits(long long mx) {
+  const double tie = (1.0 - TIE_RTOL) * (1.0 - TIE_RTOL);   // on squared norms
+  return mx > 0x7ff0000000000000ll ? mx : dbits(__longlong_as_double(mx) * tie);
+}
 
 // ------------------------------------------------------------ column-pivoted QR
 // Businger-Golub Householder QR with column pivoting of Y (m x e, ld ldy, precision T),
@@ -267,7 +275,6 @@ __device__ int block_cpqr(T* Y, int ldy, int m, int e, double eps, int* perm, do
   }
   __syncthreads();
   const double tol3z = sqrt(DBL_EPSILON);
-  const double tie = (1.0 - TIE_RTOL) * (1.0 - TIE_RTOL);   // on squared norms
   const int kmax = min(min(m, e), kstop);
   double ref = 0.0;
   int k = kmax;
@@ -278,14 +285,14 @@ __device__ int block_cpqr(T* Y, int ldy, int m, int e, double eps, int* perm, do
     const int wr = (i + 2 + blockIdx.x) % NWT, wd = (i + 3 + blockIdx.x) % NWT;
     if (warp == wp) {         // pivot: largest norm, near-ties -> lowest index
       long long mx = -1;
-      for (int j = i + lane; j < e; j += 32) mx = max(mx, dbits(vn1[j]));
+      for (int j = i + lane; j < e; j += 32) mx = max(mx, norm_bits(vn1[j]));
       for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      const long long thr = dbits(__longlong_as_double(mx) * tie);
+      const long long thr = tie_bits(mx);
       int best = e;
       for (int j = i + lane; j < e; j += 32)
-        if (dbits(vn1[j]) >= thr && j < best) best = j;
+        if (norm_bits(vn1[j]) >= thr && j < best) best = j;
       for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(0xffffffffu, best, o));
-      if (lane == 0) shi[0] = best < e ? best : i;     // i: only where a norm is not a number
+      if (lane == 0) shi[0] = best < e ? best : i;
     }
     __syncthreads();
     const int p = shi[0];
@@ -823,41 +830,44 @@ __device__ __forceinline__ void qr_bar() {
 
 __device__ __forceinline__ unsigned bits_hi(double x) { return (unsigned)((unsigned long long)dbits(x) >> 32); }
 __device__ __forceinline__ unsigned bits_lo(double x) { return (unsigned)(unsigned long long)dbits(x); }
+__device__ __forceinline__ unsigned abs_hi(double x) { return bits_hi(x) & 0x7fffffffu; }
+__device__ __forceinline__ unsigned abs_hi(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+__device__ __forceinline__ unsigned abs_lo(double x) { return bits_lo(x); }
+__device__ __forceinline__ unsigned abs_lo(float) { return 0u; }
 
-// normx = sqrt(s) of a positive s: in FP64 from the reciprocal square root (a division or square
-// root costs 6 to 10 dependent FP64 instructions of 67 cycles each)
+// normx = sqrt(s) of a sum of squares: in FP64 from the reciprocal square root (a division or square
+// root costs 6 to 10 dependent FP64 instructions of 67 cycles each).  Only a sum of exactly 0 gives
+// 0, the mark of a column without entries; one that is not finite gives NaN.
 __device__ __forceinline__ float qr_norm(float s) { return sqrtf(s); }
-__device__ __forceinline__ double qr_norm(double s) { return s > 0.0 ? s * rsqrt(s) : 0.0; }
+__device__ __forceinline__ double qr_norm(double s) { return dbits(s) == 0 ? 0.0 : s * rsqrt(s); }
 
 // The pivot of a step, chosen by one warp: among its columns at positions >= i, the largest
 // squared norm, near-ties (TIE_RTOL) to the lowest position.  Norms are compared as bit patterns
-// (an FP64 comparison is an instruction of the FP64 pipe).  Returns the position; *col the column.
+// (an FP64 comparison is an instruction of the FP64 pipe; norm_bits).  Returns the position; *col
+// the column.
 template <int CS>
 __device__ __forceinline__ int qr_pivot(const double (&n1)[CS], const int (&pos)[CS], int i, int e, int* col) {
-  const int lane = threadIdx.x & 31;
-  const double tie = (1.0 - TIE_RTOL) * (1.0 - TIE_RTOL);   // on squared norms
   unsigned hi = 0, lo = 0, best = 0xffffffffu;
 #pragma unroll
   for (int t = 0; t < CS; ++t)
-    if (pos[t] >= i && pos[t] < e) hi = max(hi, bits_hi(n1[t]));
+    if (pos[t] >= i && pos[t] < e) hi = max(hi, abs_hi(n1[t]));
   hi = __reduce_max_sync(0xffffffffu, hi);
 #pragma unroll
   for (int t = 0; t < CS; ++t)
-    if (pos[t] >= i && pos[t] < e && bits_hi(n1[t]) == hi) lo = max(lo, bits_lo(n1[t]));
+    if (pos[t] >= i && pos[t] < e && abs_hi(n1[t]) == hi) lo = max(lo, bits_lo(n1[t]));
   lo = __reduce_max_sync(0xffffffffu, lo);
-  const long long thr = dbits(__longlong_as_double(((long long)hi << 32) | lo) * tie);
+  const long long thr = tie_bits(((long long)hi << 32) | lo);
 #pragma unroll
   for (int t = 0; t < CS; ++t)
-    if (pos[t] >= i && pos[t] < e && dbits(n1[t]) >= thr) best = min(best, (unsigned)pos[t]);
+    if (pos[t] >= i && pos[t] < e && norm_bits(n1[t]) >= thr) best = min(best, (unsigned)pos[t]);
   best = __reduce_min_sync(0xffffffffu, best);
-  if (best >= (unsigned)e) best = (unsigned)i;   // only where a norm is not a number
+  if (best >= (unsigned)e) best = (unsigned)i;
   *col = 0;
 #pragma unroll
   for (int t = 0; t < CS; ++t) {
     const unsigned b = __ballot_sync(0xffffffffu, pos[t] == (int)best);
     if (b) *col = 32 * t + __ffs(b) - 1;
   }
-  (void)lane;
   return (int)best;
 }
 
@@ -1188,11 +1198,6 @@ __device__ void fast_interp(const T* Y, int ldy, int k, int e, const int* slot, 
   }
   __syncthreads();
 }
-
-__device__ __forceinline__ unsigned abs_hi(double x) { return bits_hi(x) & 0x7fffffffu; }
-__device__ __forceinline__ unsigned abs_hi(float x) { return __float_as_uint(x) & 0x7fffffffu; }
-__device__ __forceinline__ unsigned abs_lo(double x) { return bits_lo(x); }
-__device__ __forceinline__ unsigned abs_lo(float) { return 0u; }
 
 // Elimination of the last n = e - k rows and columns of the e x e block A (e <= 32 RS) with partial
 // pivoting among those rows: L, U and the multipliers in place (interchanged with their rows),
@@ -1989,7 +1994,6 @@ __device__ int wide_qr(cg::cluster_group& cl, const WideShape& W, T* Yl, int ldl
   T* yc[MS];
   double n1[MS], g2[MS];
   const double tol3z = sqrt(DBL_EPSILON);
-  const double tie = (1.0 - TIE_RTOL) * (1.0 - TIE_RTOL);
 #pragma unroll
   for (int t = 0; t < MS; ++t) {
     col[t] = 32 * (set0 + 8 * t) + lane;
@@ -2044,25 +2048,25 @@ __device__ int wide_qr(cg::cluster_group& cl, const WideShape& W, T* Yl, int ldl
     unsigned hi = 0, lo = 0;
 #pragma unroll
     for (int t = 0; t < MS; ++t)
-      if (own && pos[t] >= i && pos[t] < e) hi = max(hi, bits_hi(n1[t]));
+      if (own && pos[t] >= i && pos[t] < e) hi = max(hi, abs_hi(n1[t]));
     hi = __reduce_max_sync(0xffffffffu, hi);
 #pragma unroll
     for (int t = 0; t < MS; ++t)
-      if (own && pos[t] >= i && pos[t] < e && bits_hi(n1[t]) == hi) lo = max(lo, bits_lo(n1[t]));
+      if (own && pos[t] >= i && pos[t] < e && abs_hi(n1[t]) == hi) lo = max(lo, bits_lo(n1[t]));
     lo = __reduce_max_sync(0xffffffffu, lo);
     if (lane == 0) { red[2 * warp] = hi; red[2 * warp + 1] = lo; }
     __syncthreads();
     unsigned long long mx = 0;
 #pragma unroll
     for (int q = 0; q < 8; ++q) mx = max(mx, ((unsigned long long)red[2 * q] << 32) | red[2 * q + 1]);
-    const long long thr = dbits(__longlong_as_double((long long)mx) * tie);
+    const long long thr = tie_bits((long long)mx);
     unsigned best = 0xffffffffu, first = 0xffffffffu;
 #pragma unroll
     for (int t = 0; t < MS; ++t)
       if (own && pos[t] >= i && pos[t] < e) {
         const unsigned key = ((unsigned)pos[t] << 16) | (unsigned)col[t];
         first = min(first, key);
-        if (dbits(n1[t]) >= thr) best = min(best, key);
+        if (norm_bits(n1[t]) >= thr) best = min(best, key);
       }
     best = __reduce_min_sync(0xffffffffu, best);
     first = __reduce_min_sync(0xffffffffu, first);
@@ -2071,7 +2075,7 @@ __device__ int wide_qr(cg::cluster_group& cl, const WideShape& W, T* Yl, int ldl
     best = first = 0xffffffffu;
 #pragma unroll
     for (int q = 0; q < 8; ++q) { best = min(best, red[16 + q]); first = min(first, red[24 + q]); }
-    return best != 0xffffffffu ? best : first;               // first: only where a norm is not a number
+    return best != 0xffffffffu ? best : first;
   };
   double v[MS];
 #pragma unroll

@@ -39,3 +39,22 @@ def test_pivot_searches_stay_inside_large_blocks(kind, nx, ny, eps, precision):
     P.A.data[_entry(P.A, node, node)] = np.nan
     X = _solution(P, eps_id=eps, precision=precision)
     assert X is None or not np.isfinite(X).all()
+
+
+# The coupling of a segment's end node to its junction lies in no other block than the neighbour
+# block that the segment's ID samples: an ID that takes its column for zero loses it.  At the first
+# cut of the finest level, and where the two coarsest cuts meet: there the segment keeps every
+# unknown on the finer levels and meets the junction again in the forms of the coarse ones.
+@pytest.mark.parametrize("value", [np.nan, -np.nan, np.inf])
+@pytest.mark.parametrize("coarse", [False, True])
+@pytest.mark.parametrize("kind,nx,ny,precision", [("convdiff", 63, 63, 0), ("aniso", 255, 127, 0),
+                                                  ("convdiff", 127, 63, 1)])
+def test_neighbour_coupling_is_not_lost(kind, nx, ny, precision, coarse, value):
+    if precision == 1 and np.isinf(value):
+        pytest.skip("in FP32 an infinite norm also stands for finite entries whose squares overflow")
+    P = W.make_problem(kind, nx, seed=102, nrhs=1, ny=ny)
+    x, y = (nx // 2, ny // 2) if coarse else (15, 15)
+    i, j = x - 1 + nx * y, x + nx * y
+    P.A.data[_entry(P.A, i, j)] = value
+    X = _solution(P, eps_id=4e-7 if precision else 1e-8, precision=precision)
+    assert X is None or not np.isfinite(X).all()
