@@ -1436,8 +1436,9 @@ __host__ __device__ inline size_t sparsify_smem_small(int e, int tbytes) {
 }
 __host__ __device__ inline int sparsify_t_values(int e) { return e * e / 4 > 8 * e ? e * e / 4 : 8 * e; }
 
+// Segment of this CTA: ID, elimination of the remainder, outputs (every thread calls it).
 template <typename T, int NWT>
-__global__ void __launch_bounds__(NWT * 32, NWT == NW ? 4 : 16) sparsify_kernel(LevelDev d, int smem_bytes) {
+__device__ __forceinline__ void sparsify_segment(const LevelDev& d, int smem_bytes) {
   extern __shared__ double sm[];
   __shared__ SegCtx S;
   __shared__ double shr[NWT * 64 + 3 * 64];
@@ -1450,15 +1451,12 @@ __global__ void __launch_bounds__(NWT * 32, NWT == NW ? 4 : 16) sparsify_kernel(
   __syncthreads();
   const int e = S.e;
   const int capS = d.capS;
-  // Beside a wide kernel this one starts early: what follows both waits for both through the last CTA,
-  // which ends no sooner than the clusters do (with no such launch before it the wait is none)
-  auto leave = [&]() { if (blockIdx.x == gridDim.x - 1) pdl_wait(); };
-  if (wide_takes(d, S, sizeof(T))) return leave();     // sparsify_wide_kernel's
+  if (wide_takes(d, S, sizeof(T))) return;             // sparsify_wide_kernel's
   int* perm_out = d.perm + (size_t)sid * capS;
   if (threadIdx.x == 0) atomicMax(d.lstat + LS_EMAX, e);
   if (e == 0) {
     if (threadIdx.x == 0) { d.kk[sid] = 0; d.hs[sid] = 0; }
-    return leave();
+    return;
   }
   const size_t ld = d.ldF;
   const T* F1 = static_cast<const T*>(d.F) + (size_t)S.b1 * ld * ld;
@@ -1837,7 +1835,15 @@ __global__ void __launch_bounds__(NWT * 32, NWT == NW ? 4 : 16) sparsify_kernel(
     atomicAdd(d.flops, work_done);
     atomicAdd(d.flops + 2, (unsigned long long)((k * r + e * e) * sizeof(T) + 2 * e * sizeof(int)));
   }
-  leave();
+}
+
+// Beside a wide kernel this one starts early: what follows both waits for both through the last CTA,
+// which ends no sooner than the clusters do, whichever way its segment ended (with no such launch
+// before it the wait is none).
+template <typename T, int NWT>
+__global__ void __launch_bounds__(NWT * 32, NWT == NW ? 4 : 16) sparsify_kernel(LevelDev d, int smem_bytes) {
+  sparsify_segment<T, NWT>(d, smem_bytes);
+  if (blockIdx.x == gridDim.x - 1) pdl_wait();
 }
 
 // W = L^{-1} P A_pd and Z = A_dp U^{-1} for the 32 boundary unknowns x0 .. x0 + 31 of a parent, from
