@@ -172,6 +172,7 @@ struct spalu_factor_s {
     long long n_pre = 0, n_ok = 0;   // kernels of the graph: before the guard's node, in its body
     long long captures = 0, replays = 0, refits = 0, continued = 0;   // statistics (spalu_stats)
     std::vector<long long> n_step;   // ... and in each Arnoldi step's node
+    std::vector<SolveCaps> caps;     // [1..L] the captured solve kernels' capacities
   } sg;
   int* d_lstat = nullptr;    // [LS_N * (L + 1)] per-level counters (factor kernels)
   unsigned long long* d_flops = nullptr;   // [4 * (L + 1)] per level: algorithmic FLOPs of the sparsify
@@ -1524,23 +1525,45 @@ static spalu_status step_prepare(spalu_factor_t f, spalu_factor_s::StepGraph& G)
   }
   std::vector<int> ref(3 * (L + 1), 0);
   for (int l = 1; l <= L; ++l) {
+    const LevelDev& d = f->lev[l];
+    const SolveCaps& now = f->caps[l];
+    const int* v = &f->lstat[LS_N * l];
+    // a quarter, at least 4, but no more than the geometry allows; the forms for up to INV_MAX unknowns
+    // (level solves at 1023^2, mixed: 324 us, the general ones 634) are kept where that leaves the
+    // least headroom of 4
+    const int most[3] = {d.capS, d.sepcap, d.gp.D()};
     int lm[LS_N] = {};
-    for (int q = 0; q < 3; ++q) {
-      const int v = f->lstat[LS_N * l + q];
-      lm[q] = v + std::max(4, v / 4);
-    }
+    for (int q = 0; q < 3; ++q) lm[q] = std::max(v[q], std::min(v[q] + std::max(4, v[q] / 4), most[q]));
+    if (now.seg_team && v[0] + 4 <= INV_MAX) lm[0] = std::min(lm[0], INV_MAX);
+    if (now.sep_team && v[1] + 4 <= INV_MAX) lm[1] = std::min(lm[1], INV_MAX);
     SolveCaps c;
-    if (level_solve_caps(f->lev[l], lm, &c)) {
-      c.seg_nt = f->caps[l].seg_nt;
-      c.sep_nt = f->caps[l].sep_nt;
-      c.seg_split = f->caps[l].seg_split;
-      c.sep_split = f->caps[l].sep_split;
+    bool fits = level_solve_caps(d, lm, &c);
+    // ... also where the separator and its boundary with their headroom outgrow shared memory
+    for (int h = std::max(lm[1] - v[1], lm[2] - v[2]) / 2; fits && now.sep_team && !c.sep_team && h >= 4; h /= 2) {
+      int less[LS_N] = {lm[0], std::min(lm[1], v[1] + h), std::min(lm[2], v[2] + h)};
+      SolveCaps t;
+      if (level_solve_caps(d, less, &t) && t.sep_team) {
+        std::copy(less, less + LS_N, lm);
+        c = t;
+      }
+    }
+    if (fits) {
+      // the tuned widths and groups belong to the tuned form
+      if (c.seg_team == now.seg_team) {
+        c.seg_nt = now.seg_nt;
+        c.seg_split = now.seg_split;
+      }
+      if (c.sep_team == now.sep_team) {
+        c.sep_nt = now.sep_nt;
+        c.sep_split = now.sep_split;
+      }
       f->caps[l] = c;
     } else {
-      for (int q = 0; q < 3; ++q) lm[q] = f->lstat[LS_N * l + q];
+      for (int q = 0; q < 3; ++q) lm[q] = v[q];
     }
     for (int q = 0; q < 3; ++q) ref[3 * l + q] = lm[q];
   }
+  G.caps = f->caps;
   f->kumax = f->kumax <= 15 ? 15 : 30;       // the two leaf-sweep variants
   CUDA_TRY(cudaMemcpy(G.d_ref, ref.data(), sizeof(int) * ref.size(), cudaMemcpyHostToDevice));
   G.K = std::min(f->o.gmres_m, std::max(4, f->gmres_hint + 2));
@@ -2050,19 +2073,25 @@ spalu_status spalu_stats(spalu_factor_t f, char* json, size_t cap) {
       ksum += kk[i];
     }
     if (emax > 0) qt = std::max(qt, (double)kmax / emax);
-    char buf[640];
+    char buf[800];
     const int* ls = f->lstat.data() + LS_N * l;
-    std::snprintf(buf, sizeof buf, "%s{\"level\": %d, \"nseg\": %d, \"e_max\": %d, \"k_max\": %d, \"e_sum\": %lld, \"k_sum\": %lld, \"sep_k_max\": %d, \"passes\": %d, \"fallbacks\": %d, \"predicted\": %d, \"flops_sparsify\": %llu, \"flops_merge\": %llu, \"bytes_seg\": %llu, \"bytes_sep\": %llu, \"predictor\": %d}",
+    std::snprintf(buf, sizeof buf, "%s{\"level\": %d, \"nseg\": %d, \"e_max\": %d, \"k_max\": %d, \"e_sum\": %lld, \"k_sum\": %lld, \"sep_k_max\": %d, \"passes\": %d, \"fallbacks\": %d, \"predicted\": %d, \"flops_sparsify\": %llu, \"flops_merge\": %llu, \"bytes_seg\": %llu, \"bytes_sep\": %llu, \"predictor\": %d, \"solve_form\": [%d, %d, %d, %d]}",
                   l == 1 ? "" : ", ", l, n, emax, kmax, esum, ksum, ls[LS_KPMAX], ls[LS_PASSES],
                   ls[LS_FALLBACK], ls[LS_PREDICTED], fl[4 * l], fl[4 * l + 1], fl[4 * l + 2], fl[4 * l + 3],
-                  d.pred_mode);
+                  d.pred_mode, f->caps[l].seg_team, f->caps[l].sep_team, f->caps[l].seg_nt, f->caps[l].sep_nt);
     out += buf;
   }
   char buf[256];
   std::snprintf(buf, sizeof buf, "], \"q_tilde\": %.6f, \"step_graph\": {\"captures\": %lld, \"replays\": %lld, "
-                "\"refits\": %lld, \"continued\": %lld}", qt, f->sg.captures, f->sg.replays, f->sg.refits,
-                f->sg.continued);
+                "\"refits\": %lld, \"continued\": %lld, \"solve_forms\": [", qt, f->sg.captures, f->sg.replays,
+                f->sg.refits, f->sg.continued);
   out += buf;
+  for (size_t l = 1; l < f->sg.caps.size(); ++l) {
+    const SolveCaps& c = f->sg.caps[l];
+    std::snprintf(buf, sizeof buf, "%s[%d, %d, %d, %d]", l == 1 ? "" : ", ", c.seg_team, c.sep_team, c.seg_nt, c.sep_nt);
+    out += buf;
+  }
+  out += "]}";
   f->timer.collect();
   out += ", \"timing_ms\": {";
   bool first = true;

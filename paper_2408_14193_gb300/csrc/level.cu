@@ -41,7 +41,6 @@ constexpr int SK_CHUNK_MAX = 64;  // ... and at most, where the shared-memory bu
 constexpr int NW = 8;             // warps per CTA of the sparsify kernel (segments with e > 32)
 constexpr int NW_SMALL = 2;       // ... and for levels whose segments have at most 16 unknowns
 constexpr double TIE_RTOL = 1e-12;
-constexpr int INV_MAX = 64;       // triangular blocks up to this order are stored inverted (see below)
 constexpr int RSTAGE = 96;        // triangular blocks up to this order are staged in shared memory
 
 // ------------------------------------------------------------ Philox4x32-10 (SC'11)

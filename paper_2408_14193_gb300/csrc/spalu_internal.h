@@ -183,6 +183,10 @@ struct LevelDev {
   const float4* nstat;      // per grid node {log|A_uu|, log(|A_uu|/off), |row sum|/|A_uu|, asymmetry}
 };
 
+// Triangular blocks up to this order are stored inverted; segments and separators up to it have their
+// own forms of the level solve.
+constexpr int INV_MAX = 64;
+
 // Shared-memory capacities of the solve kernels of one level, set by the host from the
 // largest sizes the factor met at that level.
 struct SolveCaps {
