@@ -3868,7 +3868,6 @@ static void sparsify_launch(const LevelDev& d0, const LevelPlan& p, cudaStream_t
   cfg.attrs = attr;
   cfg.numAttrs = 0;
   if constexpr (sizeof(T) == 8) if (d.wide > 1) {
-    cudaFuncSetAttribute(sparsify_wide_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, d.wide_smem);
     cfg.gridDim = dim3(d.g.nseg() * d.wide);
     cfg.blockDim = dim3(256);
     cfg.dynamicSmemBytes = d.wide_smem;
@@ -3878,7 +3877,7 @@ static void sparsify_launch(const LevelDev& d0, const LevelPlan& p, cudaStream_t
     attr[0].val.clusterDim.z = 1;
     cfg.numAttrs = 1;
     note_launch();
-    cudaLaunchKernelEx(&cfg, sparsify_wide_kernel<T>, d);
+    cudaLaunchKernelEx(&cfg, smem_allowed<sparsify_wide_kernel<T>>(), d);
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
   }
@@ -3886,13 +3885,12 @@ static void sparsify_launch(const LevelDev& d0, const LevelPlan& p, cudaStream_t
   cfg.dynamicSmemBytes = smem;
   note_launch();
   auto run = [&](auto kernel, int threads) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     cfg.blockDim = dim3(threads);
     cudaLaunchKernelEx(&cfg, kernel, d, smem);
   };
-  if (d.capS <= 16) run(sparsify_kernel<T, NW_SMALL>, NW_SMALL * 32);   // two warps each, many segments per SM
-  else run(sparsify_kernel<T, NW>, NW * 32);
+  if (d.capS <= 16) run(smem_allowed<sparsify_kernel<T, NW_SMALL>>(), NW_SMALL * 32);   // two warps each, many segments per SM
+  else run(smem_allowed<sparsify_kernel<T, NW>>(), NW * 32);
 }
 
 void launch_sparsify(const LevelDev& d, const LevelPlan& p, cudaStream_t s) {
@@ -3929,7 +3927,6 @@ static void merge_launch(const LevelDev& d, const LevelPlan& p, cudaStream_t s) 
       const size_t km = std::min(p.sepcap, SIDES_MAX);
       pm = std::max(pm, (int)(sizeof(T) * (km * ((km + 7) / 8) + km) + 16 * (km + 2) + 4 * (km + 2)));
     }
-    cudaFuncSetAttribute(merge_panel_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, pm);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(np, cl);
     cfg.blockDim = dim3(256);
@@ -3943,14 +3940,13 @@ static void merge_launch(const LevelDev& d, const LevelPlan& p, cudaStream_t s) 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     note_launch();
-    cudaLaunchKernelEx(&cfg, merge_panel_kernel<T>, d);
+    cudaLaunchKernelEx(&cfg, smem_allowed<merge_panel_kernel<T>>(), d);
     if (sides) {
       int ks = std::min(p.sepcap, SIDES_MAX);
       while (!sides_fit<T>(ks)) --ks;
       const int sb = (int)sides_bytes<T>(ks);
-      cudaFuncSetAttribute(merge_sides_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sb);
       note_launch();
-      merge_sides_kernel<T><<<dim3(np, std::min((p.ldFp + 31) / 32, 48)), 256, sb, s>>>(d);
+      smem_allowed<merge_sides_kernel<T>>()<<<dim3(np, std::min((p.ldFp + 31) / 32, 48)), 256, sb, s>>>(d);
     }
   }
   note_launch();
@@ -4036,7 +4032,6 @@ static void level_solve(const LevelDev& d, const SolveCaps& sc, T* X, int nrhs, 
     const int nc = nrhs - c0 < SC ? nrhs - c0 : SC;
     T* Xc = X + (size_t)(c0 / SC) * lay.chunk;
     auto go = [&](auto kern, int n, int split, int threads, size_t smem) {
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       note_launch();
       launch_pdl(kern, dim3(n, split < nc ? split : nc), dim3(threads), smem, s, d, sc, Xc, nc, lay, bwd);
     };
@@ -4044,23 +4039,23 @@ static void level_solve(const LevelDev& d, const SolveCaps& sc, T* X, int nrhs, 
       const int n = d.g.nseg();
       if (n == 0) return;
       if (sc.seg_team) {
-        if (sc.seg_nt == 64) go(seg_team_kernel<T, 64>, n, sc.seg_split, 64, sc.seg_smem);
-        else go(seg_team_kernel<T, 256>, n, sc.seg_split, 256, sc.seg_smem);
+        if (sc.seg_nt == 64) go(smem_allowed<seg_team_kernel<T, 64>>(), n, sc.seg_split, 64, sc.seg_smem);
+        else go(smem_allowed<seg_team_kernel<T, 256>>(), n, sc.seg_split, 256, sc.seg_smem);
       } else if (sc.seg_nt == 64) {       // 2-warp CTAs: four times as many resident per SM
-        go(seg_solve_kernel<T, 64>, n, sc.seg_split, 64, sc.seg_smem);
+        go(smem_allowed<seg_solve_kernel<T, 64>>(), n, sc.seg_split, 64, sc.seg_smem);
       } else {
-        go(seg_solve_kernel<T, 256>, n, sc.seg_split, 256, sc.seg_smem);
+        go(smem_allowed<seg_solve_kernel<T, 256>>(), n, sc.seg_split, 256, sc.seg_smem);
       }
     };
     auto sep_go = [&]() {
       const int n = d.gp.nbox();
       if (sc.sep_team) {
-        if (sc.sep_nt == 64) go(sep_team_kernel<T, 64>, n, sc.sep_split, 64, sc.sep_smem);
-        else go(sep_team_kernel<T, 256>, n, sc.sep_split, 256, sc.sep_smem);
+        if (sc.sep_nt == 64) go(smem_allowed<sep_team_kernel<T, 64>>(), n, sc.sep_split, 64, sc.sep_smem);
+        else go(smem_allowed<sep_team_kernel<T, 256>>(), n, sc.sep_split, 256, sc.sep_smem);
       } else if (sc.sep_nt == 64) {
-        go(sep_solve_kernel<T, 64>, n, sc.sep_split, 64, sc.sep_smem);
+        go(smem_allowed<sep_solve_kernel<T, 64>>(), n, sc.sep_split, 64, sc.sep_smem);
       } else {
-        go(sep_solve_kernel<T, 256>, n, sc.sep_split, 256, sc.sep_smem);
+        go(smem_allowed<sep_solve_kernel<T, 256>>(), n, sc.sep_split, 256, sc.sep_smem);
       }
     };
     if (!bwd) { seg_go(); sep_go(); }

@@ -272,6 +272,23 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
+// Kernel K, allowed all the dynamic shared memory that its static part leaves of a CTA's.  The limit
+// belongs to the function, not to a launch: kernels whose launches differ in size get this one value
+// from every thread, so that a handle in one thread cannot lower it before another's launch.
+template <auto K>
+inline decltype(K) smem_allowed() {
+  static const int bytes = [] {
+    int dev = 0, most = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaFuncAttributes a{};
+    cudaFuncGetAttributes(&a, K);
+    return most - (int)a.sharedSizeBytes;
+  }();
+  cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  return K;
+}
+
 // Placement of a solve vector: element (grid node u, right-hand side c) at X[u * rs + c * cs];
 // the solve kernels take the right-hand sides in chunks of 16, chunk k at X + k * chunk.
 // Column-major (ld): {1, ld, 16 ld}; chunk-interleaved (16 values per node): {16, 1, 16 N}.
