@@ -284,10 +284,11 @@ void spalu_batch_graph_destroy(spalu_batch_t b);
 
 /* JSON summary of the last factorization: per level the segment sizes and ranks, the
  * largest separator skeleton, the number of IDs computed ("passes"), of predicted one-pass
- * IDs and of those that fell back to the adaptive schedule, and "solve_form": whether the
- * segments and the separators take the level-solve kernels for at most 64 unknowns, and the
- * threads of their CTAs (the captured step's: "step_graph", "solve_forms"); q~ (Sec. 6);
- * device bytes held.  Synchronises the factor's stream. */
+ * IDs, of those that fell back to the adaptive schedule and of segments that worked in global
+ * scratch ("scratch", see spars_ctas), and "solve_form": whether the segments and the
+ * separators take the level-solve kernels for at most 64 unknowns, and the threads of their
+ * CTAs (the captured step's: "step_graph", "solve_forms"); q~ (Sec. 6); device bytes held.
+ * Synchronises the factor's stream. */
 spalu_status spalu_stats(spalu_factor_t f, char* json, size_t cap);
 
 /* Index tables of level l (1 <= l <= L) as the last factorization left them, for parity

@@ -2075,9 +2075,9 @@ spalu_status spalu_stats(spalu_factor_t f, char* json, size_t cap) {
     if (emax > 0) qt = std::max(qt, (double)kmax / emax);
     char buf[800];
     const int* ls = f->lstat.data() + LS_N * l;
-    std::snprintf(buf, sizeof buf, "%s{\"level\": %d, \"nseg\": %d, \"e_max\": %d, \"k_max\": %d, \"e_sum\": %lld, \"k_sum\": %lld, \"sep_k_max\": %d, \"passes\": %d, \"fallbacks\": %d, \"predicted\": %d, \"flops_sparsify\": %llu, \"flops_merge\": %llu, \"bytes_seg\": %llu, \"bytes_sep\": %llu, \"predictor\": %d, \"solve_form\": [%d, %d, %d, %d]}",
+    std::snprintf(buf, sizeof buf, "%s{\"level\": %d, \"nseg\": %d, \"e_max\": %d, \"k_max\": %d, \"e_sum\": %lld, \"k_sum\": %lld, \"sep_k_max\": %d, \"passes\": %d, \"fallbacks\": %d, \"predicted\": %d, \"scratch\": %d, \"flops_sparsify\": %llu, \"flops_merge\": %llu, \"bytes_seg\": %llu, \"bytes_sep\": %llu, \"predictor\": %d, \"solve_form\": [%d, %d, %d, %d]}",
                   l == 1 ? "" : ", ", l, n, emax, kmax, esum, ksum, ls[LS_KPMAX], ls[LS_PASSES],
-                  ls[LS_FALLBACK], ls[LS_PREDICTED], fl[4 * l], fl[4 * l + 1], fl[4 * l + 2], fl[4 * l + 3],
+                  ls[LS_FALLBACK], ls[LS_PREDICTED], ls[LS_SCRATCH], fl[4 * l], fl[4 * l + 1], fl[4 * l + 2], fl[4 * l + 3],
                   d.pred_mode, f->caps[l].seg_team, f->caps[l].sep_team, f->caps[l].seg_nt, f->caps[l].sep_nt);
     out += buf;
   }

@@ -1597,6 +1597,7 @@ __device__ __forceinline__ void sparsify_segment(const LevelDev& d, int smem_byt
     if (threadIdx.x == 0) { atomicOr(d.err, ERR_CAPACITY); d.kk[sid] = 0; d.hs[sid] = 0; }
     return;
   }
+  if (!in_smem && threadIdx.x == 0) atomicAdd(d.lstat + LS_SCRATCH, 1);
   // B staged once (all loads in flight) for the near rows, every sketch pass, the probe and
   // the error test; otherwise each reads the frontal blocks through the neighbour table
   if (bstage) {

@@ -47,7 +47,7 @@ constexpr int PRED_OFF_B2 = PRED_OFF_W2 + PRED_NOUT * PRED_NHID;
 // predictor modes of a factorization
 enum { PRED_OFF = 0, PRED_RECORD = 1, PRED_PREDICT = 2 };
 // per-level counters (int) written by the factor kernels
-enum { LS_EMAX = 0, LS_KPMAX = 1, LS_DPMAX = 2, LS_PASSES = 3, LS_FALLBACK = 4, LS_PREDICTED = 5, LS_N = 8 };
+enum { LS_EMAX = 0, LS_KPMAX = 1, LS_DPMAX = 2, LS_PASSES = 3, LS_FALLBACK = 4, LS_PREDICTED = 5, LS_SCRATCH = 6, LS_N = 8 };
 
 // Inference copy of the network: feature standardisation and bfloat16 parameters
 // (W1 64x16 row-major | b1 | W2 2x64 | b2).
@@ -164,7 +164,8 @@ struct LevelDev {
   int sketch_tc;    // sketch products G B_F on the tensor cores (mixed path only)
   unsigned long long seed;
   int* err;
-  int* lstat;       // [LS_N] counters of this level (maxima of e, kp, |dP|; ID passes, ...)
+  int* lstat;       // [LS_N] counters of this level (maxima of e, kp, |dP|; ID passes, ...; segments
+                    // whose sparsification worked in global scratch)
   unsigned long long* flops;   // [4] of this level: algorithmic FLOPs of the sparsification and of
                                // the separator eliminations (work.cuh), and the bytes of the
                                // segment factors (T, transformed block, remainder LU, pivots)
