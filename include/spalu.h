@@ -78,9 +78,10 @@ typedef struct {
   int spars_ctas;             /* performance only: the sparsification's per-segment shared
                                  memory is cut to what lets min(spars_ctas, ceil(segments of
                                  the level / SMs)) segments (at most what the register file
-                                 holds) run at once on an SM; a segment that does not fit
-                                 keeps its sketch rows in global memory (results agree up to
-                                 rounding).  A level with at most one segment per SM gets
+                                 holds) run at once on an SM, but not below what a segment of
+                                 40 unknowns needs (fewer run at once then, whatever the value
+                                 here); a segment that does not fit works in global memory
+                                 (results agree up to rounding).  A level with at most one segment per SM gets
                                  200 KB (room for larger sketch chunks and the staged
                                  neighbour block).  0 = size for the largest segment the
                                  geometry allows.  Default 4. */

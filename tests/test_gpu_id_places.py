@@ -36,3 +36,15 @@ def test_scratch_agrees_with_shared_memory(kind, eps, precision, tol):
     for a, b in zip(level[1], level[4]):
         assert (a["k_max"], a["k_sum"], a["e_sum"], a["passes"]) == (b["k_max"], b["k_sum"], b["e_sum"], b["passes"]), (a, b)
     assert_close(X[4], X[1], tol, f"{kind} precision {precision}")
+
+
+def test_segments_of_up_to_40_unknowns_keep_their_place():
+    """However many segments per SM are asked for (1984 at the finest level, 976 of up to 31 unknowns)."""
+    import torch
+    from paper_2408_14193_gb300 import Factor, NestedDissection
+    dev = torch.device("cuda:0")
+    P = W.make_problem("diffusion", 511, seed=63, nrhs=1)
+    f = Factor(NestedDissection(511), eps_id=1e-8, symmetric=1, spars_ctas=16)
+    f.factor(*[torch.from_numpy(a).to(dev) for a in (P.A.indptr, P.A.indices, P.A.data)])
+    few = [lv for lv in f.stats()["levels"] if lv["e_max"] <= 40]
+    assert max(lv["nseg"] for lv in few) == 1984 and all(lv["scratch"] == 0 for lv in few), few
