@@ -1122,8 +1122,8 @@ __global__ void __launch_bounds__(RWPB * 32) leaf_rows_kernel(LeafDev d, double*
   rows_load_L(lr, 0, l, lv);                           // the factor's: overlaps the preceding kernel
   pdl_enter();
   // rows l, l + 16, ... of the right-hand sides (backward: of A_Id x_d, the terms of a row in the
-  // order of the CSR columns; a coefficient of 0 may stand for a side outside the grid, and then
-  // the row's own node, which exists, is read and not used)
+  // order of the CSR columns; a coefficient of 0 may stand for a side outside the grid, so nothing is
+  // read for it)
 #pragma unroll 1
   for (int blk = 0; blk < RNB + 1; ++blk) {
     const int jr = 16 * blk + l, j = min(jr, NI - 1);

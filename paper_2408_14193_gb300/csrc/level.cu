@@ -1421,7 +1421,8 @@ __global__ void __launch_bounds__(1024) seg_order_kernel(const int* cnt, int nse
   for (int s = threadIdx.x; s < nseg; s += blockDim.x) order[atomicAdd(&start[key(cnt[s])], 1)] = s;
 }
 
-constexpr int WIDE_EMAX = 512;
+constexpr int WIDE_EMAX = 512;    // rows that wide_interp keeps in registers; shared memory ends before
+                                  // (sparsify_wide_plan)
 // Segments of at most 32 unknowns go to a cluster from this many entries of B; larger ones always do.
 // Measured per level, one CTA / cluster: e 31 with 4000 entries 291 / 322 us, e 31 with 9000 312 / 291,
 // e 46 with 4500 457 / 406, e 267 without neighbours (the last separator) 12.9 ms / 0.74 ms.
@@ -3779,8 +3780,11 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 16) sep_solve_kernel(Level
 
 // Clusters per segment and their shared memory (0: none): FP64, levels of more than 16 unknowns per
 // side whose segments leave SMs idle.  Up to 8 CTAs a segment, two per SM at most; one per SM where
-// there is room for that, with all of the shared memory (segments of up to about 290 unknowns), else
-// half of it (about 160).
+// there is room for that, with all of the shared memory, else half of it.  Largest segments by
+// wide_bytes at the default h0 and p, without neighbours / with six sides of neighbours: 8 CTAs with
+// all of it (up to 19 segments on 152 SMs) 267 / 257 symmetric, 256 / 251 with both halves of B; with
+// half of it (up to 38) 171 / 162 and 161 / 155; 4 CTAs (up to 76) 138 / 131 and 128 / 123; 2 (up to
+// 152) 99 / 97 and 94 / 91.  A larger segment stays with one CTA.
 void sparsify_wide_plan(const LevelPlan& p, LevelDev* d) {
   d->wide = d->wide_smem = 0;
   const int n = p.g.nseg(), sms = sm_count();
