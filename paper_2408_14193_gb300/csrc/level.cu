@@ -234,9 +234,10 @@ __device__ __forceinline__ T bval_q(const LevelDev& d, const SegCtx& S, const T*
 
 // non-negative doubles order like their bit patterns
 __device__ __forceinline__ long long dbits(double x) { return __double_as_longlong(x); }
-// ... a squared norm that is not a number (of either sign) above them all: its column becomes the
-// pivot, and what is not a number reaches R, T and the solution instead of passing for a zero column
-__device__ __forceinline__ long long norm_bits(double x) { return dbits(x) & 0x7fffffffffffffffll; }
+// ... one that is not a number above them all once its sign is gone: squared norms are kept without
+// it, such a column becomes the pivot, and what is not a number reaches R, T and the solution instead
+// of passing for a zero column
+__device__ __forceinline__ double unsign(double x) { return __longlong_as_double(dbits(x) & 0x7fffffffffffffffll); }
 // the smallest pattern that ties with the largest squared norm mx (a pattern)
 __device__ __forceinline__ long long tie_bits(long long mx) {
   const double tie = (1.0 - TIE_RTOL) * (1.0 - TIE_RTOL);   // on squared norms
@@ -268,7 +269,7 @@ __device__ int block_cpqr(T* Y, int ldy, int m, int e, double eps, int* perm, do
     for (int r = lane; r < m; r += 32) { T v = Y[r + (size_t)ldy * j]; s += v * v; }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {
-      vn1[j] = (double)s;
+      vn1[j] = unsign((double)s);
       vn2[j] = (double)s;
     }
   }
@@ -284,12 +285,12 @@ __device__ int block_cpqr(T* Y, int ldy, int m, int e, double eps, int* perm, do
     const int wr = (i + 2 + blockIdx.x) % NWT, wd = (i + 3 + blockIdx.x) % NWT;
     if (warp == wp) {         // pivot: largest norm, near-ties -> lowest index
       long long mx = -1;
-      for (int j = i + lane; j < e; j += 32) mx = max(mx, norm_bits(vn1[j]));
+      for (int j = i + lane; j < e; j += 32) mx = max(mx, dbits(vn1[j]));
       for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       const long long thr = tie_bits(mx);
       int best = e;
       for (int j = i + lane; j < e; j += 32)
-        if (norm_bits(vn1[j]) >= thr && j < best) best = j;
+        if (dbits(vn1[j]) >= thr && j < best) best = j;
       for (int o = 16; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(0xffffffffu, best, o));
       if (lane == 0) shi[0] = best < e ? best : i;
     }
@@ -381,7 +382,7 @@ __device__ int block_cpqr(T* Y, int ldy, int m, int e, double eps, int* perm, do
       for (int r = i + 1 + lane; r < m; r += 32) { double v = (double)Y[r + (size_t)ldy * j]; s += v * v; }
       for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
       if (lane == 0) {
-        vn1[j] = s;
+        vn1[j] = unsign(s);
         vn2[j] = s;
       }
     }
@@ -842,23 +843,22 @@ __device__ __forceinline__ double qr_norm(double s) { return dbits(s) == 0 ? 0.0
 
 // The pivot of a step, chosen by one warp: among its columns at positions >= i, the largest
 // squared norm, near-ties (TIE_RTOL) to the lowest position.  Norms are compared as bit patterns
-// (an FP64 comparison is an instruction of the FP64 pipe; norm_bits).  Returns the position; *col
-// the column.
+// (an FP64 comparison is an instruction of the FP64 pipe).  Returns the position; *col the column.
 template <int CS>
 __device__ __forceinline__ int qr_pivot(const double (&n1)[CS], const int (&pos)[CS], int i, int e, int* col) {
   unsigned hi = 0, lo = 0, best = 0xffffffffu;
 #pragma unroll
   for (int t = 0; t < CS; ++t)
-    if (pos[t] >= i && pos[t] < e) hi = max(hi, abs_hi(n1[t]));
+    if (pos[t] >= i && pos[t] < e) hi = max(hi, bits_hi(n1[t]));
   hi = __reduce_max_sync(0xffffffffu, hi);
 #pragma unroll
   for (int t = 0; t < CS; ++t)
-    if (pos[t] >= i && pos[t] < e && abs_hi(n1[t]) == hi) lo = max(lo, bits_lo(n1[t]));
+    if (pos[t] >= i && pos[t] < e && bits_hi(n1[t]) == hi) lo = max(lo, bits_lo(n1[t]));
   lo = __reduce_max_sync(0xffffffffu, lo);
   const long long thr = tie_bits(((long long)hi << 32) | lo);
 #pragma unroll
   for (int t = 0; t < CS; ++t)
-    if (pos[t] >= i && pos[t] < e && norm_bits(n1[t]) >= thr) best = min(best, (unsigned)pos[t]);
+    if (pos[t] >= i && pos[t] < e && dbits(n1[t]) >= thr) best = min(best, (unsigned)pos[t]);
   best = __reduce_min_sync(0xffffffffu, best);
   if (best >= (unsigned)e) best = (unsigned)i;
   *col = 0;
@@ -929,7 +929,7 @@ __device__ int fast_cpqr(T* Y, int ldy, int m, int e, double eps, int* perm, int
       for (int t = 0; t < CS; ++t) {
         T s = T(0);
         for (int w = 0; w < QW; ++w) s += part[w * EC + lane + 32 * t];
-        n1[t] = lane + 32 * t < e ? (double)s : 0.0;
+        n1[t] = lane + 32 * t < e ? unsign((double)s) : 0.0;
         g2[t] = tol3z * n1[t];
       }
       int pc;
@@ -1090,7 +1090,7 @@ __device__ int fast_cpqr(T* Y, int ldy, int m, int e, double eps, int* perm, int
             if (t < cs) {
               double q = part2[lane + 32 * t];
               for (int w = 1; w < QW; ++w) q += part2[w * EC + lane + 32 * t];
-              if (act[t]) { n1[t] = q; g2[t] = tol3z * q; }
+              if (act[t]) { n1[t] = unsign(q); g2[t] = tol3z * q; }
             }
           }
           int pn;
@@ -2055,11 +2055,11 @@ __device__ int wide_qr(cg::cluster_group& cl, const WideShape& W, T* Yl, int ldl
     unsigned hi = 0, lo = 0;
 #pragma unroll
     for (int t = 0; t < MS; ++t)
-      if (own && pos[t] >= i && pos[t] < e) hi = max(hi, abs_hi(n1[t]));
+      if (own && pos[t] >= i && pos[t] < e) hi = max(hi, bits_hi(n1[t]));
     hi = __reduce_max_sync(0xffffffffu, hi);
 #pragma unroll
     for (int t = 0; t < MS; ++t)
-      if (own && pos[t] >= i && pos[t] < e && abs_hi(n1[t]) == hi) lo = max(lo, bits_lo(n1[t]));
+      if (own && pos[t] >= i && pos[t] < e && bits_hi(n1[t]) == hi) lo = max(lo, bits_lo(n1[t]));
     lo = __reduce_max_sync(0xffffffffu, lo);
     if (lane == 0) { red[2 * warp] = hi; red[2 * warp + 1] = lo; }
     __syncthreads();
@@ -2073,7 +2073,7 @@ __device__ int wide_qr(cg::cluster_group& cl, const WideShape& W, T* Yl, int ldl
       if (own && pos[t] >= i && pos[t] < e) {
         const unsigned key = ((unsigned)pos[t] << 16) | (unsigned)col[t];
         first = min(first, key);
-        if (norm_bits(n1[t]) >= thr) best = min(best, key);
+        if (dbits(n1[t]) >= thr) best = min(best, key);
       }
     best = __reduce_min_sync(0xffffffffu, best);
     first = __reduce_min_sync(0xffffffffu, first);
@@ -2094,7 +2094,7 @@ __device__ int wide_qr(cg::cluster_group& cl, const WideShape& W, T* Yl, int ldl
   }
   gather_sum(v, nullptr);
 #pragma unroll
-  for (int t = 0; t < MS; ++t) { n1[t] = v[t]; g2[t] = tol3z * v[t]; }
+  for (int t = 0; t < MS; ++t) { n1[t] = unsign(v[t]); g2[t] = tol3z * v[t]; }
   unsigned key = choose(0);
   int k = kmax;
   for (int i = 0; i < kmax; ++i) {
@@ -2193,7 +2193,7 @@ __device__ int wide_qr(cg::cluster_group& cl, const WideShape& W, T* Yl, int ldl
       gather_sum(v, nullptr);
 #pragma unroll
       for (int t = 0; t < MS; ++t)
-        if (own && val[t] && pos[t] > i) { n1[t] = v[t]; g2[t] = tol3z * v[t]; }
+        if (own && val[t] && pos[t] > i) { n1[t] = unsign(v[t]); g2[t] = tol3z * v[t]; }
     }
     key = choose(i + 1);       // its barriers also order the update before the next products
   }
