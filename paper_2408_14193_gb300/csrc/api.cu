@@ -1528,14 +1528,17 @@ static spalu_status step_prepare(spalu_factor_t f, spalu_factor_s::StepGraph& G)
     const LevelDev& d = f->lev[l];
     const SolveCaps& now = f->caps[l];
     const int* v = &f->lstat[LS_N * l];
-    // a quarter, at least 4, but no more than the geometry allows; the forms for up to INV_MAX unknowns
-    // (level solves at 1023^2, mixed: 324 us, the general ones 634) are kept where that leaves the
-    // least headroom of 4
-    const int most[3] = {d.capS, d.sepcap, d.gp.D()};
+    // headroom of a quarter, at least 4; where that would lose the forms for up to INV_MAX unknowns
+    // (level solves at 1023^2, mixed: 324 us, the general ones 634) no more than the geometry allows,
+    // and none past INV_MAX where that leaves the least headroom
     int lm[LS_N] = {};
-    for (int q = 0; q < 3; ++q) lm[q] = std::max(v[q], std::min(v[q] + std::max(4, v[q] / 4), most[q]));
-    if (now.seg_team && v[0] + 4 <= INV_MAX) lm[0] = std::min(lm[0], INV_MAX);
-    if (now.sep_team && v[1] + 4 <= INV_MAX) lm[1] = std::min(lm[1], INV_MAX);
+    for (int q = 0; q < 3; ++q) lm[q] = v[q] + std::max(4, v[q] / 4);
+    auto keep = [&](int q, int most) {
+      if (lm[q] > INV_MAX) lm[q] = std::max(v[q], std::min(lm[q], most));
+      if (v[q] + 4 <= INV_MAX) lm[q] = std::min(lm[q], INV_MAX);
+    };
+    if (now.seg_team) keep(0, d.capS);
+    if (now.sep_team) keep(1, d.sepcap);
     SolveCaps c;
     bool fits = level_solve_caps(d, lm, &c);
     // ... also where the separator and its boundary with their headroom outgrow shared memory
